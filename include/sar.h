@@ -173,7 +173,8 @@ typedef struct sar_plan_info {
     int64_t n_pixels;           /* image size in complex64 values */
     int32_t n_tiles;            /* pixel tiles of 1024 reconstruction points (slots) */
     int32_t window_bins;        /* bins staged per (tile, chirp, Rx) */
-    int32_t pulses_per_block;   /* chirps staged per pipeline step */
+    int32_t pulses_per_block;   /* chirps staged per pipeline step (calls that take the pair path, see
+                                   sar_backproject, stage as many as fit when this is the largest block) */
     int32_t bp_ctas;            /* persistent backprojection grid size */
     double bins_per_metre;      /* a1 = mu N_fft / (c fs) */
     double cycles_per_bin;      /* f0 / (c a1) */
@@ -256,6 +257,12 @@ int sar_range_spectrum(sar_plan *plan, const void *beat_dev, int32_t M,
  * gets no contribution from the call (its value is written as 0, or left
  * unchanged when accumulating) and the call is flagged SAR_EBOUNDS too: its
  * interpolation index would leave the staged bin window.
+ * Large calls go through a workspace of the plan that holds the profiles as
+ * interpolation pairs (16 bytes per bin of max_pulses chirps, part of
+ * device_bytes; a plan goes without it where it would take over 1 GiB or a
+ * sixteenth of the free memory, or where its HBM budget would not hold the
+ * buffers allocated later).  A call on another stream than the previous one
+ * waits for it.
  */
 int sar_backproject(sar_plan *plan, const void *prof_dev, int32_t M,
                     const double *q_tx_dev, const double *q_rx_dev,

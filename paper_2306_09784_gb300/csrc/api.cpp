@@ -19,8 +19,19 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846264338327950288;
 constexpr size_t kBpSmemTarget = 110 * 1024;  // two CTAs per SM
+constexpr size_t kBpSmemTarget3 = 73 * 1024;  // three
 constexpr size_t kBpSmemMax = 227 * 1024;
 constexpr int kMaxPulsesPerBlock = 32;
+// Dynamic shared memory of the pair kernel with two and three CTAs per SM
+// (228 KB per SM, 1 KB of each CTA reserved).
+constexpr size_t kPairSmem[2] = {113 * 1024, 75 * 1024};
+// Largest workspace of interpolation pairs a plan keeps.
+constexpr size_t kPairBytesMax = size_t(1) << 30;
+// Calls of at least this many windows (pixel tiles x chirps x Rx, 6.7e7 updates,
+// ~50 us) take the pair kernel.  Its extra launch and the pairs it writes cost
+// ~5 us, its pixel loop saves ~8 %: 131072 windows in 139 us against 144 us,
+// 4096 windows in 32 us against 29 us.
+constexpr long long kPairMinWindows = 65536;
 
 }  // namespace
 
@@ -39,6 +50,20 @@ struct sar_plan {
     int num_sms = 0, ctas_per_sm = 0, G = 0, minb = 2;
     size_t partial_slots = 0;  // partial-sum tile slots allocated
     float fd_max = 0.f;
+    // backprojection from interpolation pairs (backproject_pairs.cu): the
+    // workspace, when the plan has one, and the launch that goes with rg and
+    // minb.  mb_cap: chirps per pipeline block at most (explicit blocks only)
+    float4 *d_pairs = nullptr, *d_rx = nullptr, *d_zero = nullptr;
+    float *d_o2max = nullptr;
+    int zero_len = 0;
+    unsigned long long *d_call = nullptr;
+    unsigned epoch = 0;
+    // the stream and the end of the last call that used the workspace: a call
+    // on another stream waits for it
+    cudaStream_t pair_stream = nullptr;
+    cudaEvent_t pair_done = nullptr;
+    size_t pair_smem = 0;
+    int pair_G = 0, mb_cap = kMaxPulsesPerBlock;
     // device memory owned by the plan
     float *d_wr = nullptr;
     float2 *d_tw = nullptr;
@@ -47,6 +72,7 @@ struct sar_plan {
     int *d_out = nullptr;
     TileInfo *d_tiles = nullptr;
     float2 *d_partial = nullptr;
+    int *d_arrived = nullptr;
     int *d_err = nullptr;
     double *d_means = nullptr;  // sar_doppler_offsets: mean positions and velocity
     // tables of the split-transform range compression (when supported)
@@ -75,6 +101,7 @@ struct sar_plan {
         int *d_out = nullptr;
         TileInfo *d_tiles = nullptr;
         float2 *d_partial = nullptr;
+        int *d_arrived = nullptr;  // pair kernel: arrivals of split tiles (after the partial sums)
     };
     std::vector<Tiling> tilings;
     int tile_w = 0;
@@ -210,13 +237,34 @@ void free_plan(sar_plan *pl) {
     cudaDeviceSynchronize();
     for (void *p : pl->allocs) cudaFree(p);
     if (pl->s_copy) cudaStreamDestroy(pl->s_copy);
-    for (cudaEvent_t e : {pl->ev_start, pl->ev_chunk[0], pl->ev_chunk[1], pl->ev_traj})
+    for (cudaEvent_t e : {pl->ev_start, pl->ev_chunk[0], pl->ev_chunk[1], pl->ev_traj, pl->pair_done})
         if (e) cudaEventDestroy(e);
     delete pl;
 }
 
 // Largest of 4, 3, 2, 1 that divides the Rx count.
 int default_rx_group(int R) { return (R % 4 == 0) ? 4 : (R % 3 == 0) ? 3 : (R % 2 == 0) ? 2 : 1; }
+
+// Chirps of the largest block whose staging fits minb CTAs per SM.
+int largest_block(const sar_plan *pl, int L, int minb) {
+    const size_t budget = minb == 3 ? kBpSmemTarget3 : kBpSmemTarget;
+    int Mb = kMaxPulsesPerBlock;
+    while (Mb > 1 && bp_smem_bytes(Mb, pl->p.n_rx, L, pl->fp16) > budget) --Mb;
+    return Mb;
+}
+
+// The pair kernel's launch for this Rx group and register budget (the current
+// tiling); false where it does not fit.
+bool pair_launch(const sar_plan *pl, int rg, int minb, size_t *smem, int *G) {
+    *smem = std::max(kPairSmem[minb - 2], bp_pairs_min_smem(pl->p.n_rx, pl->L));
+    int occ = 0;
+    if (*smem > kBpSmemMax || bp_pairs_prepare(rg, pl->p.n_rx, *smem, minb, &occ) != cudaSuccess || occ < 1) {
+        cudaGetLastError();
+        return false;
+    }
+    *G = pl->num_sms * std::min(occ, minb);
+    return (size_t)*G * (size_t)(pl->n_tiles / *G + 2) <= pl->partial_slots;
+}
 
 // Validate and install a backprojection launch shape; the plan is unchanged
 // on failure.
@@ -238,6 +286,13 @@ int apply_launch(sar_plan *pl, int rg, int minb, int Mb) {
     const int G = pl->num_sms * occ;
     // split-tile slots of the worst case (one pulse block per tile)
     if ((size_t)G * (size_t)(pl->n_tiles / G + 2) > pl->partial_slots) return SAR_EINVAL;
+    size_t pair_smem = 0;
+    int pair_G = 0;
+    if (pl->d_pairs && !pair_launch(pl, rg, minb, &pair_smem, &pair_G)) return SAR_EINVAL;
+    pl->pair_smem = pair_smem;
+    pl->pair_G = pair_G;
+    // the largest block of the copying kernel stands for as many as fit
+    pl->mb_cap = Mb >= largest_block(pl, pl->L, minb) ? kMaxPulsesPerBlock : Mb;
     pl->rg = rg;
     pl->minb = minb;
     pl->Mb = Mb;
@@ -552,8 +607,11 @@ int install_tiling(sar_plan *pl, const HostTiles &ht, int tw, int L) {
     if (!rc) rc = upload(pl, ht.tiles, &t.d_tiles);
     if (!rc) {
         void *q = nullptr;
-        rc = dev_alloc(pl, t.partial_slots * kTilePx * sizeof(float2), &q);
+        const size_t sums = t.partial_slots * kTilePx * sizeof(float2), counts = (size_t)t.n_tiles * 8 * sizeof(int);
+        rc = dev_alloc(pl, sums + counts, &q);
         t.d_partial = (float2 *)q;
+        t.d_arrived = (int *)((char *)q + sums);
+        if (!rc && cudaMemset(t.d_arrived, 0, counts) != cudaSuccess) rc = SAR_ECUDA;
     }
     if (rc) return rc;  // what was allocated is freed with the plan
     pl->tilings.push_back(t);
@@ -569,6 +627,7 @@ void use_tiling(sar_plan *pl, const sar_plan::Tiling &t) {
     pl->d_out = t.d_out;
     pl->d_tiles = t.d_tiles;
     pl->d_partial = t.d_partial;
+    pl->d_arrived = t.d_arrived;
 }
 
 // Switch a Cartesian plan to tiles tw pixels wide (16, 32 or 64), building
@@ -605,6 +664,58 @@ int plan_retile(sar_plan *pl, int tw) {
     use_tiling(pl, prev);
     apply_launch(pl, rg, minb, Mb0);
     return SAR_EINVAL;
+}
+
+size_t profile_bytes(const sar_plan *pl, int M) {
+    const size_t rows = (size_t)M * pl->p.n_rx;
+    if (pl->fp16) return ((rows * 4 + 255) & ~size_t(255)) + rows * pl->n_bins * 4;
+    return rows * pl->n_bins * 8;
+}
+
+// Workspace of the pair kernel: 16 bytes per bin of max_pulses chirps, twice
+// an FP32 profile buffer.  A plan goes without (and uses the copying kernel)
+// where it would take more than 1 GiB or a sixteenth of the free memory, or
+// where an HBM budget would then no longer hold the buffers that
+// sar_form_image_host and sar_plan_set_tile_shape allocate later.
+void add_pair_workspace(sar_plan *pl) {
+    const size_t rows = (size_t)pl->p.max_pulses * pl->p.n_rx;
+    const size_t bytes = rows * pl->n_bins * sizeof(float4);
+    const size_t geo = rows * sizeof(float4) + (size_t)pl->p.max_pulses * sizeof(float);
+    size_t free_b = 0, total_b = 0;
+    if (bytes > kPairBytesMax || rows > (size_t)1 << 30 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+        bytes > free_b / 16) {
+        cudaGetLastError();
+        return;
+    }
+    // zeros for windows outside the crop, as long as any tiling's window: a
+    // 64 x 16 or 16 x 64 tile is at most 2.1 times as wide as a 32 x 32 one
+    const int zero_len = (int)(2.25 * pl->L) + 16;
+    if (pl->budget) {
+        const size_t M = (size_t)pl->p.max_pulses, R = (size_t)pl->p.n_rx;
+        const size_t host = M * R * pl->p.n_samples * 8 + M * 20 + M * R * 16 + profile_bytes(pl, (int)M) +
+                            (size_t)pl->n_pixels * 8 + 8 * 256;
+        const size_t tiles = (size_t)pl->n_pixels / 512 + 4 * (size_t)pl->n_tiles + 64;
+        const size_t retile = pl->tile_w ? 2 * tiles * (kTilePx * 20 + sizeof(TileInfo)) +
+                                               12 * (size_t)pl->num_sms * kTilePx * 8 + 8 * 256
+                                         : 0;
+        if (pl->used + bytes + geo + (size_t)zero_len * 16 + 1024 + host + retile > pl->budget) return;
+    }
+    // one block: call words, zeros, Rx offsets and their largest squares
+    const size_t rx_o = 256 + (size_t)zero_len * sizeof(float4);
+    void *small = nullptr, *pairs = nullptr;
+    if (dev_alloc(pl, rx_o + geo, &small) || dev_alloc(pl, bytes, &pairs) ||
+        cudaMemset(small, 0, rx_o) != cudaSuccess ||
+        cudaEventCreateWithFlags(&pl->pair_done, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    pl->d_pairs = (float4 *)pairs;
+    pl->d_call = (unsigned long long *)small;
+    pl->d_zero = (float4 *)((char *)small + 256);
+    pl->zero_len = zero_len;
+    pl->d_rx = (float4 *)((char *)small + rx_o);
+    pl->d_o2max = (float *)(pl->d_rx + rows);
+    if (!pair_launch(pl, pl->rg, pl->minb, &pl->pair_smem, &pl->pair_G)) pl->d_pairs = nullptr;
 }
 
 int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t budget, sar_plan **out) {
@@ -746,19 +857,13 @@ int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t bud
         free_plan(pl);
         return rc;
     }
+    add_pair_workspace(pl);
     recall_shape(pl);
     *out = pl;
     return SAR_OK;
 }
 
-size_t profile_bytes(const sar_plan *pl, int M) {
-    const size_t rows = (size_t)M * pl->p.n_rx;
-    if (pl->fp16) return ((rows * 4 + 255) & ~size_t(255)) + rows * pl->n_bins * 4;
-    return rows * pl->n_bins * 8;
-}
-
 bool aligned(const void *p, size_t a) { return ((uintptr_t)p % a) == 0; }
-
 
 // Split-kernel job from the general kernel's arguments and the plan's tables.
 void split_args(const sar_plan *pl, const RcArgs &a, RcSplitArgs *b) {
@@ -897,11 +1002,69 @@ bool set_launch(const sar_plan *pl, BpArgs &a, float2 *partial, size_t slots) {
     return (size_t)a.G * (size_t)a.seg_max <= slots;
 }
 
+bool use_pairs(const sar_plan *pl, int M) {
+    return pl->d_pairs && pl->L <= pl->zero_len &&
+           (long long)pl->n_tiles * M * pl->p.n_rx >= kPairMinWindows;
+}
+
+// Backprojection from interpolation pairs of a call's arguments a.
+int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
+    BpPairArgs pa{};
+    a.blocks_per_tile = (a.M + kPairUnit - 1) / kPairUnit;
+    a.units = (long long)a.n_tiles * a.blocks_per_tile;
+    a.G = (int)std::min<long long>(pl->pair_G, a.units);
+    const long long per = (a.units + a.G - 1) / a.G;
+    a.seg_max = (int)((per - 1) / a.blocks_per_tile) + 2;
+    a.partial = pl->d_partial;
+    if ((size_t)a.G * (size_t)a.seg_max > pl->partial_slots) return SAR_EINVAL;  // cannot happen
+    pa.b = a;
+    pa.pairs = pl->d_pairs;
+    pa.zero = pl->d_zero;
+    pa.rx = pl->d_rx;
+    pa.o2max = pl->d_o2max;
+    pa.call = pl->d_call;
+    pa.arrived = pl->d_arrived;
+    pa.div_blk = ((1ull << 32) + (unsigned)a.Mb - 1) / (unsigned)a.Mb;
+    pa.smem_bytes = (unsigned)pl->pair_smem;
+    pa.mb_cap = pl->mb_cap;
+    ExpandArgs e{};
+    e.prof = a.prof;
+    e.scales = a.prof_scale;
+    e.q_tx = a.q_tx;
+    e.q_rx = a.q_rx;
+    e.pairs = pl->d_pairs;
+    e.rx = pl->d_rx;
+    e.o2max = pl->d_o2max;
+    e.call = pl->d_call;
+    e.epoch = ++pl->epoch;
+    e.rows = a.M * a.R;
+    e.R = a.R;
+    e.n_bins = a.n_bins;
+    e.cb_k = a.cb_k;
+    e.inv_kappa = a.inv_kappa;
+    const BpLaunch l{pl->rg, pl->fp16, pl->pair_smem, pl->minb};
+    DeviceGuard dg(pl->device);
+    if (!dg.ok) return SAR_ECUDA;
+    // (a captured call is ordered by its graph)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return SAR_ECUDA;
+    if (cap == cudaStreamCaptureStatusNone && s != pl->pair_stream &&
+        cudaStreamWaitEvent(s, pl->pair_done, 0) != cudaSuccess)
+        return SAR_ECUDA;
+    if (launch_backproject_pairs(pa, e, l, s) != cudaSuccess) return SAR_ECUDA;
+    if (cap == cudaStreamCaptureStatusNone) {
+        if (cudaEventRecord(pl->pair_done, s) != cudaSuccess) return SAR_ECUDA;
+        pl->pair_stream = s;
+    }
+    return SAR_OK;
+}
+
 int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const double *q_rx, const float *fd,
               void *image, int accumulate, cudaStream_t s, int m0 = 0, int M_tot = 0,
               void *image_out = nullptr) {
     BpArgs a = common_bp_args(pl, prof, M, q_tx, q_rx, fd, image, accumulate, m0, M_tot);
     a.image_out = (float2 *)image_out;
+    if (use_pairs(pl, M)) return bp_launch_pairs(pl, a, s);
     if (!set_launch(pl, a, pl->d_partial, pl->partial_slots)) return SAR_EINVAL;  // cannot happen
     BpLaunch l{pl->rg, pl->fp16, pl->bp_smem, pl->minb};
     DeviceGuard dg(pl->device);
@@ -998,7 +1161,7 @@ int sar_plan_get_info(const sar_plan *pl, sar_plan_info *info) {
     i.n_tiles = pl->n_tiles;
     i.window_bins = pl->L;
     i.pulses_per_block = pl->Mb;
-    i.bp_ctas = pl->G;
+    i.bp_ctas = pl->d_pairs ? pl->pair_G : pl->G;
     i.bins_per_metre = pl->a1;
     i.cycles_per_bin = pl->beta;
     i.device_bytes = pl->used;
@@ -1635,7 +1798,7 @@ int sar_plan_autotune(sar_plan *pl, const void *prof_dev, int32_t M, const doubl
         int rg1 = 0;
         for (int g = rg0 - 1; g >= 1 && !rg1; --g)
             if (R % g == 0) rg1 = g;
-        const size_t budgets[2] = {kBpSmemTarget, 73 * 1024};
+        const size_t budgets[2] = {kBpSmemTarget, kBpSmemTarget3};
         for (int rg : {rg0, rg1}) {
             if (rg < 1) continue;
             for (int minb = 2; minb <= 3; ++minb) {
@@ -1814,6 +1977,9 @@ int sar_plan_check_errors(sar_plan *pl) {
     int h[4] = {0, 0, 0, 0};
     if (cudaMemcpy(h, pl->d_err, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess) return SAR_ECUDA;
     if (cudaMemset(pl->d_err, 0, sizeof(h)) != cudaSuccess) return SAR_ECUDA;
+    if (h[0] & kErrStall)  // a launch gave up: arrivals of its split tiles are void
+        for (const sar_plan::Tiling &t : pl->tilings)
+            if (cudaMemset(t.d_arrived, 0, (size_t)t.n_tiles * 8 * sizeof(int)) != cudaSuccess) return SAR_ECUDA;
     return h[0] ? SAR_EBOUNDS : SAR_OK;
 }
 

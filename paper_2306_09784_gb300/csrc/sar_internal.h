@@ -21,6 +21,7 @@ constexpr double kMaxRange = 1.0e6;
 // Bits of the device error flag (any bit set: SAR_EBOUNDS).
 constexpr int kErrGeometry = 1;      // non-finite or out-of-range antenna geometry
 constexpr int kErrDopplerBound = 2;  // |f_doppler(p)| beyond the plan's bound, or not finite
+constexpr int kErrStall = 4;         // a bounded wait of a kernel ran out (never expected)
 
 // Range compression output modes.
 enum RcMode { kRcProfileF32 = 0, kRcProfileF16 = 1, kRcSpectrum = 2 };
@@ -168,6 +169,38 @@ struct BpLaunch {
     size_t smem;  // dynamic shared memory bytes
     int minb;     // CTAs per SM the kernel's registers are sized for (2 or 3)
 };
+
+// Backprojection from interpolation pairs (backproject_pairs.cu).
+constexpr int kPairUnit = 2;  // pulses per work unit
+struct BpPairArgs {
+    BpArgs b;                  // units, blocks_per_tile: in units of kPairUnit pulses; Mb: pulses per
+                               // aligned run that shares the loop choice; prof unused
+    unsigned long long div_blk;  // ceil(2^32 / Mb)
+    const float4 *pairs;       // [M R][n_bins] (A, D) of bins crop_lo ... (the last one of a row unused)
+    const float4 *zero;        // L zero entries
+    const float4 *rx;          // [M R] Rx offset (o_x, o_y, |o|^2, 0)
+    const float *o2max;        // [M] largest |o|^2 of the pulse
+    const unsigned long long *call;  // low words: FP32 bits of the call's largest |o|; any o_y
+    int *arrived;              // [n_tiles][8] warps done with a split tile's pixels, zero between launches
+    unsigned smem_bytes;       // dynamic shared memory of the launch
+    int mb_cap;                // chirps per pipeline block at most
+};
+struct ExpandArgs {
+    const void *prof;          // profile samples (float2 or half2)
+    const float *scales;       // FP16 scales
+    const double *q_tx, *q_rx;
+    float4 *pairs;
+    float4 *rx;
+    float *o2max;
+    unsigned long long *call;
+    unsigned epoch;            // the plan's call number
+    int rows, R, n_bins;
+    float2 cb_k;
+    float inv_kappa;
+};
+size_t bp_pairs_min_smem(int R, int L);
+cudaError_t bp_pairs_prepare(int rg, int R, size_t smem, int minb, int *ctas_per_sm);
+cudaError_t launch_backproject_pairs(const BpPairArgs &pa, const ExpandArgs &e, const BpLaunch &l, cudaStream_t s);
 
 size_t bp_smem_bytes(int Mb, int R, int L, bool fp16);
 cudaError_t bp_prepare(bool fp16, int rg, size_t smem);  // sets function attributes

@@ -32,6 +32,7 @@ constexpr size_t kPairBytesMax = size_t(1) << 30;
 // ~5 us, its pixel loop saves ~8 %: 131072 windows in 139 us against 144 us,
 // 4096 windows in 32 us against 29 us.
 constexpr long long kPairMinWindows = 65536;
+constexpr int kMinBlockWindows = 16;
 
 }  // namespace
 
@@ -1065,11 +1066,21 @@ int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const d
     BpArgs a = common_bp_args(pl, prof, M, q_tx, q_rx, fd, image, accumulate, m0, M_tot);
     a.image_out = (float2 *)image_out;
     if (use_pairs(pl, M)) return bp_launch_pairs(pl, a, s);
+    // a small call's blocks are cut so that every CTA has work (several blocks
+    // each, so that their counts differ little), but keep kMinBlockWindows
+    // windows: a block's set-up is ~3 us, 16 windows' pixel loop ~1 us
+    const long long fill = (long long)pl->n_tiles * M / (2ll * pl->G);
+    const int small = (int)std::max<long long>(fill, (kMinBlockWindows + a.R - 1) / a.R);
+    if (small < a.Mb && pl->mb_cap == kMaxPulsesPerBlock) {  // (an explicit block stays)
+        a.Mb = small;
+        a.blocks_per_tile = (M + a.Mb - 1) / a.Mb;
+        a.units = (long long)a.n_tiles * a.blocks_per_tile;
+    }
     if (!set_launch(pl, a, pl->d_partial, pl->partial_slots)) return SAR_EINVAL;  // cannot happen
     BpLaunch l{pl->rg, pl->fp16, pl->bp_smem, pl->minb};
     DeviceGuard dg(pl->device);
     if (!dg.ok) return SAR_ECUDA;
-    return launch_backproject(a, l, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
+    return launch_backproject(a, l, pl->d_arrived, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
 }  // namespace
@@ -1111,7 +1122,7 @@ int backproject_with_scratch(sar_plan *pl, const void *prof, int M, const double
     BpLaunch l{pl->rg, pl->fp16, pl->bp_smem, pl->minb};
     DeviceGuard dg(pl->device);
     if (!dg.ok) return SAR_ECUDA;
-    return launch_backproject(a, l, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
+    return launch_backproject(a, l, nullptr, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
 }  // namespace sar

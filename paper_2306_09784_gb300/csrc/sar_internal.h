@@ -205,7 +205,9 @@ cudaError_t launch_backproject_pairs(const BpPairArgs &pa, const ExpandArgs &e, 
 size_t bp_smem_bytes(int Mb, int R, int L, bool fp16);
 cudaError_t bp_prepare(bool fp16, int rg, size_t smem);  // sets function attributes
 int bp_occupancy(bool fp16, int rg, size_t smem, int minb, int *ctas_per_sm);
-cudaError_t launch_backproject(const BpArgs &a, const BpLaunch &l, cudaStream_t s);
+// arrived: zeroed counters (8 per tile) to sum split tiles in the same launch;
+// null: by a fix-up launch.
+cudaError_t launch_backproject(const BpArgs &a, const BpLaunch &l, int *arrived, cudaStream_t s);
 cudaError_t bp_batch_prepare(int rg, bool fp16, size_t smem, int *ctas_per_sm);
 // host_jobs: the class's jobs in host memory (the same as c.jobs), passed as
 // parameters when there are at most kParamJobs; null to read c.jobs.

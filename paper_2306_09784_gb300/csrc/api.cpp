@@ -32,7 +32,10 @@ constexpr size_t kPairBytesMax = size_t(1) << 30;
 // ~5 us, its pixel loop saves ~8 %: 131072 windows in 139 us against 144 us,
 // 4096 windows in 32 us against 29 us.
 constexpr long long kPairMinWindows = 65536;
-constexpr int kMinBlockWindows = 16;
+// Set-up of a pulse block of the copying kernel, in windows' time (~1 us, 12 of
+// ~70 ns): 128 x 128 x 256 x 1 frame 24.6 us at blocks of 16 or 32 chirps, 28.7
+// at 24, where the last CTAs of a second round run alone.
+constexpr int kBlockSetup = 12;
 
 }  // namespace
 
@@ -1066,14 +1069,23 @@ int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const d
     BpArgs a = common_bp_args(pl, prof, M, q_tx, q_rx, fd, image, accumulate, m0, M_tot);
     a.image_out = (float2 *)image_out;
     if (use_pairs(pl, M)) return bp_launch_pairs(pl, a, s);
-    // a small call's blocks are cut so that every CTA has work (several blocks
-    // each, so that their counts differ little), but keep kMinBlockWindows
-    // windows: a block's set-up is ~3 us, 16 windows' pixel loop ~1 us
-    const long long fill = (long long)pl->n_tiles * M / (2ll * pl->G);
-    const int small = (int)std::max<long long>(fill, (kMinBlockWindows + a.R - 1) / a.R);
-    if (small < a.Mb && pl->mb_cap == kMaxPulsesPerBlock) {  // (an explicit block stays)
-        a.Mb = small;
-        a.blocks_per_tile = (M + a.Mb - 1) / a.Mb;
+    // a call too small for the pair kernel cuts its pulse blocks so that the
+    // CTAs' counts of them even out: the block that minimises, in windows'
+    // time, the longest CTA (a block's set-up is worth kBlockSetup windows)
+    // plus half a window per share of a split tile.  (An explicit block stays.)
+    if (pl->mb_cap == kMaxPulsesPerBlock) {
+        long long best = INT64_MAX;
+        int mb = a.Mb;
+        for (int b = a.Mb; b >= 1; --b) {
+            const long long per_tile = (M + b - 1) / b, rounds = (a.n_tiles * per_tile + pl->G - 1) / pl->G;
+            const long long cost = 2 * rounds * ((long long)b * a.R + kBlockSetup) + per_tile;
+            if (cost < best) {
+                best = cost;
+                mb = b;
+            }
+        }
+        a.Mb = mb;
+        a.blocks_per_tile = (M + mb - 1) / mb;
         a.units = (long long)a.n_tiles * a.blocks_per_tile;
     }
     if (!set_launch(pl, a, pl->d_partial, pl->partial_slots)) return SAR_EINVAL;  // cannot happen

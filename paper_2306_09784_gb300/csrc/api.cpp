@@ -82,6 +82,10 @@ struct sar_plan {
     // tables of the split-transform range compression (when supported)
     bool rc_split = false;
     float2 *d_rc_pre = nullptr, *d_rc_twd = nullptr;
+    // and of the band kernel (rc_band != 0)
+    unsigned rc_band = 0;
+    float4 *d_rc_pre2 = nullptr, *d_rc_cmb = nullptr;
+    float2 *d_rc_twd2 = nullptr;
     // staging buffers of sar_form_image_host
     void *s_beat = nullptr;
     float *s_waz = nullptr;
@@ -839,7 +843,47 @@ int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t bud
             }
     }
 
+    // band kernel: the same input rotations by thread of a row (thread
+    // 16 (n2 os / 2 + s / 2) + b holds n = n2 + D (16 a + b) of s and s + 1), the
+    // inter-pass twiddles and the output coefficients
+    std::vector<float4> rc_pre2, rc_cmb;
+    std::vector<float2> rc_twd2;
+    pl->rc_band = pl->rc_split ? rc_band_mask(p.n_samples, p.os, pl->crop_lo, pl->crop_hi) : 0;
+    if (pl->rc_band) {
+        const int N = p.n_samples, D = N / 256, ho = p.os / 2, RT = 16 * D * ho;
+        rc_pre2.resize((size_t)16 * RT);
+        for (int a = 0; a < 16; ++a)
+            for (int t = 0; t < RT; ++t) {
+                const int g = t / 16, n = g / ho + D * (16 * a + t % 16), s = 2 * (g % ho);
+                const float2 u = rc_pre[(size_t)s * N + n], v = rc_pre[(size_t)(s + 1) * N + n];
+                rc_pre2[(size_t)a * RT + t] = make_float4(u.x, v.x, u.y, v.y);
+            }
+        auto unit = [&](long long num, long long den, double more) {
+            const double t = pl->sign * 2.0 * kPi * ((double)(num % den) / (double)den + more);
+            return make_float2((float)std::cos(t), (float)std::sin(t));
+        };
+        rc_twd2.resize(256);
+        for (int k1 = 0; k1 < 16; ++k1)
+            for (int b = 0; b < 16; ++b) rc_twd2[k1 * 16 + b] = unit((long long)b * k1, 256, 0.0);
+        const int kp0 = pl->crop_lo / 2, np = pl->crop_hi / 2 - kp0 + 1;
+        rc_cmb.resize((size_t)D * np);
+        for (int d = 0; d < D; ++d)
+            for (int i = 0; i < np; ++i) {
+                float2 u[2];
+                for (int e = 0; e < 2; ++e) {
+                    const int k = 2 * (kp0 + i) + e;
+                    double cyc = (double)k * pl->beta;
+                    cyc -= std::floor(cyc);
+                    u[e] = unit((long long)d * (k / p.os), N, cyc);
+                }
+                rc_cmb[(size_t)d * np + i] = make_float4(u[0].x, u[1].x, u[0].y, u[1].y);
+            }
+    }
+
     rc = upload(pl, wr, &pl->d_wr);
+    if (!rc && pl->rc_band) rc = upload(pl, rc_pre2, &pl->d_rc_pre2);
+    if (!rc && pl->rc_band) rc = upload(pl, rc_twd2, &pl->d_rc_twd2);
+    if (!rc && pl->rc_band) rc = upload(pl, rc_cmb, &pl->d_rc_cmb);
     if (!rc && pl->rc_split) rc = upload(pl, rc_pre, &pl->d_rc_pre);
     if (!rc && pl->rc_split) rc = upload(pl, rc_twd, &pl->d_rc_twd);
     if (!rc) rc = upload(pl, tw, &pl->d_tw);
@@ -885,6 +929,10 @@ void split_args(const sar_plan *pl, const RcArgs &a, RcSplitArgs *b) {
     b->crop_lo = pl->crop_lo;
     b->crop_hi = pl->crop_hi;
     b->n_bins = pl->n_bins;
+    b->band = pl->rc_band;
+    b->pre2 = pl->d_rc_pre2;
+    b->twd2 = pl->d_rc_twd2;
+    b->cmb = pl->d_rc_cmb;
 }
 
 // General-kernel arguments of range compression of pulses [m0, m0 + M) of a
@@ -924,7 +972,7 @@ int rc_launch_part(sar_plan *pl, const void *beat, int m0, int M, int M_tot, con
     const RcArgs a = rc_args(pl, beat, m0, M, M_tot, w_az, out, mode);
     DeviceGuard dg(pl->device);
     if (!dg.ok) return SAR_ECUDA;
-    if (pl->rc_split && mode != kRcSpectrum) {
+    if (pl->rc_split) {
         RcSplitArgs b{};
         split_args(pl, a, &b);
         return launch_range_compress_split(b, pl->sign, mode, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
@@ -1594,11 +1642,11 @@ int sar_batch_commit(sar_batch *b, void *stream) {
             c.n = 0;
             c.off = placed + b->n_rcc;
             c.groups = 0;
-            const int rpc = kSplitThreads / (ji.a.N2 * ji.a.os);
+            const int rpc = rc_rows_per_group(ji.a);
             for (size_t q = i; q < b->rc.size(); ++q) {
                 const sar_batch::RcJob &jq = b->rc[q];
                 if (!jq.split || done[q] || jq.sign != ji.sign || jq.mode != ji.mode || jq.a.N2 != ji.a.N2 ||
-                    jq.a.os != ji.a.os)
+                    jq.a.os != ji.a.os || (jq.a.band != 0) != (ji.a.band != 0))
                     continue;
                 done[q] = 1;
                 b->h_rjobs[placed] = jq.a;

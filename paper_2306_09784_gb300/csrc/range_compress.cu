@@ -611,7 +611,14 @@ __global__ void __launch_bounds__(kSplitThreads, 2) range_compress_split(RcSplit
         // across the row's threads: X = sub-transform k mod os at q = k / os,
         // times the per-bin rotation and w_sar
         const float g_az = (a.w_az != nullptr && active) ? __ldg(a.w_az + row / a.R) : 1.f;
-        if (MODE == kRcProfileF32) {
+        if (MODE == kRcSpectrum) {  // every bin, as it is
+            if (active) {
+                float2 *out = reinterpret_cast<float2 *>(a.out) + row * (long long)(N * os);
+#pragma unroll 4
+                for (int k = rem; k < N * os; k += RT) out[k] = xrow[(k & (os - 1)) * REG + (k >> sh_os)];
+            }
+            __syncthreads();  // the regions are rewritten by the next row
+        } else if (MODE == kRcProfileF32) {
             if (active) {
                 float2 *out = reinterpret_cast<float2 *>(a.out) + row * (long long)a.n_bins - a.crop_lo;
                 for (int k = a.crop_lo + rem; k <= a.crop_hi; k += RT) {
@@ -659,6 +666,275 @@ __global__ void __launch_bounds__(kSplitThreads, 2) range_compress_split(RcSplit
     for (long long g = blockIdx.x; g < n_groups; g += gridDim.x) {
         // L2 prefetch of the row this thread group handles next (one 128-byte
         // line per thread)
+        const long long gn = g + gridDim.x;
+        if constexpr (BATCH) {
+            if (gn < n_groups) {
+                long long gnl = gn;
+                const RcSplitArgs &an = tab.jobs[split_job(tab, gnl)];
+                const long long nrow = gnl * RPC + lrow;
+                if (nrow < an.rows && rem * 16 < N)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(an.beat + nrow * (long long)N + rem * 16));
+            }
+            long long gl = g;
+            const RcSplitArgs aj = tab.jobs[split_job(tab, gl)];
+            group(aj, gl);
+        } else {
+            const long long nrow = gn * RPC + lrow;
+            if (nrow < a0.rows && rem * 16 < N)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(a0.beat + nrow * (long long)N + rem * 16));
+            group(a0, g);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Band kernel: profiles whose cropped bins span at most 256 os bins, N = 256 D
+// samples (D = 1, 2), os >= 4.  With n = n2 + D n1 and bins k = os Q + s,
+//     S[os Q + s] = sum_{n2<D} W_N^{n2 Q} Y_{n2,s}[Q mod 256],
+//     Y_{n2,s}[q] = sum_{n1<256} (w_r[n] x[n] W^{n s}) W_256^{n1 q},
+// so D os transforms of 256 = 16 x 16 points replace the os transforms of N
+// points of the kernel above, and what the D-fold sum costs falls on the
+// cropped bins only (619 of 4096 on the headline frame).  A group of 16
+// threads runs the two transforms (n2, s), (n2, s + 1) in the two lanes of
+// packed FP32 (planar: real and imaginary parts of the pair), which halves the
+// arithmetic instructions without any swaps: a pass of 16-point DFTs, twiddles,
+// one exchange inside the half-warp, a second pass.  Its outputs in the band go
+// to shared memory; the row's threads then sum them over n2 with the per-bin
+// rotation folded into the twiddles and store each bin pair.
+// Bound by the load/store path (70 % of its wavefronts at 38 % issue).  Against
+// the kernel above, rows x bins: 8192 x 265 of N = 256, os 4 (FP32): 29.0 -> 19.6
+// us; 16384 x 512 of N = 256, os 8 (FP16): 101 -> 75; 16384 x 259 of N = 512, os
+// 4: 70 -> 63; 4096 x 499 of N = 512, os 8: 38.6 -> 32.8.  At N = 1024 (D = 4) a
+// thread's samples lie 32 bytes apart and their loads take a third of the path:
+// 8192 x 637 72 -> 77 us (89 us with the rows staged by cp.async), so that size
+// stays with the kernel above; at os = 2 the two are equal.
+// ---------------------------------------------------------------------------
+constexpr int kBandPairs = 4;  // bin pairs a thread keeps for the FP16 scale
+
+__host__ __device__ constexpr int band_region(int os) {
+    // 16 rows of 17 float4 (conflict-free transpose); the output stage reads
+    // 2 / os of a phase's eight lanes from each of os / 2 regions
+    return 272 + (os == 4 ? 4 : os == 8 ? 2 : os == 16 ? 1 : 0);
+}
+
+struct Planar {  // two complex values: (re0, re1), (im0, im1)
+    float2 r, i;
+};
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+
+// Butterfly a + w b, a - w b, w = exp(SGN j pi E / 8), E in [0, 8).
+template <int SGN, int E>
+__device__ __forceinline__ void bfly_planar(Planar &a, Planar &b) {
+    const Planar x = a, y = b;
+    if (E == 0) {
+        a.r = add2(x.r, y.r);
+        a.i = add2(x.i, y.i);
+        b.r = sub2(x.r, y.r);
+        b.i = sub2(x.i, y.i);
+    } else if (E == 4) {  // +-j y
+        if (SGN > 0) {
+            a.r = sub2(x.r, y.i);
+            a.i = add2(x.i, y.r);
+            b.r = add2(x.r, y.i);
+            b.i = sub2(x.i, y.r);
+        } else {
+            a.r = add2(x.r, y.i);
+            a.i = sub2(x.i, y.r);
+            b.r = sub2(x.r, y.i);
+            b.i = add2(x.i, y.r);
+        }
+    } else {
+        constexpr float c = cos_pi16(2 * E);
+        constexpr float sn = (SGN > 0 ? 1.0f : -1.0f) * (E <= 4 ? cos_pi16(8 - 2 * E) : cos_pi16(2 * E - 8));
+        a.r = fma2(dup2(c), y.r, fma2(dup2(-sn), y.i, x.r));
+        a.i = fma2(dup2(sn), y.r, fma2(dup2(c), y.i, x.i));
+        b.r = fma2(dup2(-c), y.r, fma2(dup2(sn), y.i, x.r));
+        b.i = fma2(dup2(-sn), y.r, fma2(dup2(-c), y.i, x.i));
+    }
+}
+template <int SGN, int H, int T = 0>
+__device__ __forceinline__ void stage_planar(Planar *v) {
+    if constexpr (T < H) {
+#pragma unroll
+        for (int s = 0; s < 16; s += 2 * H) bfly_planar<SGN, T * 8 / H>(v[s + T], v[s + T + H]);
+        stage_planar<SGN, H, T + 1>(v);
+    }
+}
+// 16-point DFT of both lanes, natural order in and out.
+template <int SGN>
+__device__ __forceinline__ void dft16_planar(Planar *v) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int j = bitrev(i, 4);
+        if (i < j) {
+            const Planar t = v[i];
+            v[i] = v[j];
+            v[j] = t;
+        }
+    }
+    stage_planar<SGN, 1>(v);
+    stage_planar<SGN, 2>(v);
+    stage_planar<SGN, 4>(v);
+    stage_planar<SGN, 8>(v);
+}
+
+template <int SGN, int MODE, int D, bool BATCH>
+__global__ void __launch_bounds__(kSplitThreads, 2) range_compress_band(RcSplitArgs a0, RcSplitBatch tab,
+                                                                        long long n_groups) {
+    constexpr int N = 256 * D;
+    extern __shared__ __align__(16) float4 bbuf[];  // [16 thread groups][REG]
+    __shared__ float row_max[kSplitThreads / 32];
+    const int os = a0.os, ho = os >> 1;  // the same for every job of a launch
+    const int sh_ho = 31 - __clz(ho);
+    const int REG = band_region(os);
+    const int RT = 16 * D * ho;          // threads per row
+    const int RPC = kSplitThreads / RT;  // rows per CTA
+    const int lrow = threadIdx.x / RT;
+    const int rem = threadIdx.x - lrow * RT;
+    const int n2 = (rem >> 4) >> sh_ho;  // group (n2, s pair): rem / 16 = n2 ho + s / 2
+    const int b = rem & 15;
+    float4 *xb = bbuf + (threadIdx.x >> 4) * REG;  // this group's region
+    const float4 *yrow = bbuf + lrow * D * ho * REG;
+
+    auto group = [&](const RcSplitArgs &a, long long gl) {
+        const long long row = gl * RPC + lrow;
+        const bool active = row < a.rows;
+        const float2 *x = a.beat + (active ? row : 0) * (long long)N + n2 + D * b;
+        const float4 *pre = a.pre2 + rem;  // [a][thread of the row]: (re, re), (im, im) of s, s + 1
+        Planar v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const float2 xv = active ? __ldg(x + 16 * D * i) : make_float2(0.f, 0.f);
+            const float4 t = __ldg(pre + i * RT);
+            v[i].r = make_float2(fmaf(xv.x, t.x, -xv.y * t.z), fmaf(xv.x, t.y, -xv.y * t.w));
+            v[i].i = make_float2(fmaf(xv.x, t.z, xv.y * t.x), fmaf(xv.x, t.w, xv.y * t.y));
+        }
+        dft16_planar<SGN>(v);
+        // twiddles W_256^(b k1), then element (k1, b) at 17 k1 + b
+        xb[b] = make_float4(v[0].r.x, v[0].r.y, v[0].i.x, v[0].i.y);
+#pragma unroll
+        for (int k1 = 1; k1 < 16; ++k1) {
+            const float2 w = __ldg(a.twd2 + k1 * 16 + b);
+            const float2 wr = dup2(w.x), wi = dup2(w.y), nwi = dup2(-w.y);
+            const float2 r = fma2(v[k1].r, wr, mul2(v[k1].i, nwi));
+            const float2 i = fma2(v[k1].r, wi, mul2(v[k1].i, wr));
+            xb[17 * k1 + b] = make_float4(r.x, r.y, i.x, i.y);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const float4 e = xb[17 * b + j];
+            v[j].r = make_float2(e.x, e.y);
+            v[j].i = make_float2(e.z, e.w);
+        }
+        dft16_planar<SGN>(v);
+        __syncwarp();
+        // Y[q], q = b + 16 k2, of the k2 that the band reaches
+#pragma unroll
+        for (int k2 = 0; k2 < 16; ++k2)
+            if ((a.band >> k2) & 1) xb[b + 16 * k2] = make_float4(v[k2].r.x, v[k2].r.y, v[k2].i.x, v[k2].i.y);
+        __syncthreads();
+
+        // bins 2 kp, 2 kp + 1: s pair kp mod os / 2 at Q = kp / (os / 2)
+        const float g_az = (a.w_az != nullptr && active) ? __ldg(a.w_az + row / a.R) : 1.f;
+        const int kp0 = a.crop_lo >> 1, np = (a.crop_hi >> 1) - kp0 + 1;
+        auto value = [&](int i) {
+            const int kp = kp0 + i;
+            const float4 *y = yrow + (kp & (ho - 1)) * REG + ((kp >> sh_ho) & 255);
+            const float4 *c = a.cmb + i;
+            float2 r = make_float2(0.f, 0.f), im = r;
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                const float4 e = y[d * ho * REG], t = __ldg(c + d * np);
+                const float2 er = make_float2(e.x, e.y), ei = make_float2(e.z, e.w);
+                const float2 tr = make_float2(t.x, t.y), ti = make_float2(t.z, t.w);
+                r = fma2(er, tr, fma2(make_float2(-e.z, -e.w), ti, r));
+                im = fma2(er, ti, fma2(ei, tr, im));
+            }
+            return make_float4(r.x, im.x, r.y, im.y);
+        };
+        // place of bin 0, and whether a bin pair (at even bins) can be one store
+        const long long first = row * (long long)a.n_bins - a.crop_lo;
+        constexpr int kSample = MODE == kRcProfileF32 ? 8 : 4;
+        const bool even =
+            ((reinterpret_cast<uintptr_t>(a.out) + (uintptr_t)(first * kSample)) & (2 * kSample - 1)) == 0;
+        auto store = [&](int i, float4 u, float g) {
+            const int k = 2 * (kp0 + i);
+            const bool lo = k >= a.crop_lo, hi = k + 1 <= a.crop_hi;
+            if (MODE == kRcProfileF32) {
+                float2 *out = reinterpret_cast<float2 *>(a.out) + first + k;
+                if (even && lo && hi) {
+                    *reinterpret_cast<float4 *>(out) = make_float4(g * u.x, g * u.y, g * u.z, g * u.w);
+                } else {
+                    if (lo) out[0] = make_float2(g * u.x, g * u.y);
+                    if (hi) out[1] = make_float2(g * u.z, g * u.w);
+                }
+            } else {
+                __half2 *out = reinterpret_cast<__half2 *>(a.out) + first + k;
+                const __half2 h0 = __floats2half2_rn(g * u.x, g * u.y), h1 = __floats2half2_rn(g * u.z, g * u.w);
+                if (even && lo && hi) {
+                    uint2 p;
+                    p.x = *reinterpret_cast<const uint32_t *>(&h0);
+                    p.y = *reinterpret_cast<const uint32_t *>(&h1);
+                    *reinterpret_cast<uint2 *>(out) = p;
+                } else {
+                    if (lo) out[0] = h0;
+                    if (hi) out[1] = h1;
+                }
+            }
+        };
+        if (MODE == kRcProfileF32) {
+            if (active)
+                for (int i = rem; i < np; i += RT) store(i, value(i), g_az);
+            __syncthreads();  // the regions are rewritten by the next row
+        } else {
+            float4 keep[kBandPairs];
+            float mx = 0.f;
+            auto peak = [&](int i, float4 u) {  // only bins inside the crop count
+                const int k = 2 * (kp0 + i);
+                if (k >= a.crop_lo) mx = fmaxf(mx, fmaxf(fabsf(g_az * u.x), fabsf(g_az * u.y)));
+                if (k + 1 <= a.crop_hi) mx = fmaxf(mx, fmaxf(fabsf(g_az * u.z), fabsf(g_az * u.w)));
+            };
+            if (active) {
+#pragma unroll
+                for (int q = 0; q < kBandPairs; ++q) {
+                    const int i = rem + q * RT;
+                    if (i < np) {
+                        keep[q] = value(i);
+                        peak(i, keep[q]);
+                    }
+                }
+                for (int i = rem + kBandPairs * RT; i < np; i += RT) peak(i, value(i));
+            }
+            // row maximum: within the warp's lanes of the row, then across the
+            // row's warps (RT >= 32) through shared memory
+            const int span = RT < 32 ? RT : 32;
+            for (int o = span >> 1; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            if (RT > 32) {
+                if ((threadIdx.x & 31) == 0) row_max[threadIdx.x >> 5] = mx;
+                __syncthreads();
+                const int w0 = (lrow * RT) >> 5;
+                for (int w = 0; w < (RT >> 5); ++w) mx = fmaxf(mx, row_max[w0 + w]);
+            }
+            if (active) {
+                const float scale = mx > 0.f ? mx * (1.0f / 16384.0f) : 1.0f;
+                const float inv = g_az / scale;
+                if (rem == 0) a.scales[row] = scale;
+#pragma unroll
+                for (int q = 0; q < kBandPairs; ++q) {
+                    const int i = rem + q * RT;
+                    if (i < np) store(i, keep[q], inv);
+                }
+                for (int i = rem + kBandPairs * RT; i < np; i += RT) store(i, value(i), inv);
+            }
+            __syncthreads();  // the regions and row_max are rewritten by the next row
+        }
+    };
+
+    for (long long g = blockIdx.x; g < n_groups; g += gridDim.x) {
+        // L2 prefetch of the row this thread handles next (one 128-byte line per thread)
         const long long gn = g + gridDim.x;
         if constexpr (BATCH) {
             if (gn < n_groups) {
@@ -729,19 +1005,42 @@ cudaError_t launch_rc(const RcArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+template <int SGN, int MODE, bool BATCH>
+const void *band_kernel(int D) {
+    return D == 2 ? (const void *)range_compress_band<SGN, MODE, 2, BATCH>
+                  : (const void *)range_compress_band<SGN, MODE, 1, BATCH>;
+}
+template <int SGN, int MODE, bool BATCH>
+const void *split_kernel(int N2) {
+    return N2 == 32   ? (const void *)range_compress_split<SGN, MODE, 32, BATCH>
+           : N2 == 16 ? (const void *)range_compress_split<SGN, MODE, 16, BATCH>
+                      : (const void *)range_compress_split<SGN, MODE, 8, BATCH>;
+}
+
 template <int SGN, int MODE>
 cudaError_t launch_split(const RcSplitArgs &a, const RcSplitBatch &tab, long long groups, cudaStream_t s) {
-    auto kern = tab.jobs ? (a.N2 == 32   ? range_compress_split<SGN, MODE, 32, true>
-                            : a.N2 == 16 ? range_compress_split<SGN, MODE, 16, true>
-                                         : range_compress_split<SGN, MODE, 8, true>)
-                         : (a.N2 == 32   ? range_compress_split<SGN, MODE, 32, false>
-                            : a.N2 == 16 ? range_compress_split<SGN, MODE, 16, false>
-                                         : range_compress_split<SGN, MODE, 8, false>);
-    const int rpc = kSplitThreads / (a.N2 * a.os);
-    const long long n_groups = tab.jobs ? groups : (a.rows + rpc - 1) / rpc;
+    const void *kern;
+    size_t smem;
+    int rpc;  // rows per CTA
+    bool band = false;
+    if constexpr (MODE != kRcSpectrum) band = a.band != 0;
+    if (band) {
+        if constexpr (MODE != kRcSpectrum) {
+            const int D = a.N2 / 8;
+            kern = tab.jobs ? band_kernel<SGN, MODE, true>(D) : band_kernel<SGN, MODE, false>(D);
+        }
+        smem = (size_t)(kSplitThreads / 16) * band_region(a.os) * sizeof(float4);
+    } else {
+        if constexpr (MODE == kRcSpectrum)
+            kern = split_kernel<SGN, MODE, false>(a.N2);
+        else
+            kern = tab.jobs ? split_kernel<SGN, MODE, true>(a.N2) : split_kernel<SGN, MODE, false>(a.N2);
+        // one region per sub-transform of the CTA (66 KB at N2 = 32)
+        smem = (size_t)(kSplitThreads / a.N2) * split_region(a.N2, a.os) * sizeof(float2);
+    }
+    rpc = rc_rows_per_group(a);
+    long long n_groups = tab.jobs ? groups : (a.rows + rpc - 1) / rpc;
     if (n_groups == 0) return cudaSuccess;
-    // one region per sub-transform of the CTA (66 KB at N2 = 32)
-    const size_t smem = (size_t)(kSplitThreads / a.N2) * split_region(a.N2, a.os) * sizeof(float2);
     int dev = 0, sms = 0, occ = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -749,11 +1048,26 @@ cudaError_t launch_split(const RcSplitArgs &a, const RcSplitBatch &tab, long lon
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSplitThreads, smem) != cudaSuccess || occ < 1)
         return cudaErrorInvalidConfiguration;
     const long long grid = std::min<long long>(n_groups, (long long)sms * occ);
-    kern<<<(unsigned)grid, kSplitThreads, smem, s>>>(a, tab, n_groups);
-    return cudaGetLastError();
+    RcSplitArgs arg = a;
+    RcSplitBatch t = tab;
+    void *params[] = {&arg, &t, &n_groups};
+    return cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(kSplitThreads), params, smem, s);
 }
 
 }  // namespace
+
+int rc_rows_per_group(const RcSplitArgs &a) { return kSplitThreads / (a.N2 * a.os); }
+
+// The band kernel's mask of 16-value blocks of Y, or 0 where the kernel does not
+// apply: at most 256 values of Q (else a block of Y serves several), sizes where
+// it is the faster one (see the kernel).
+unsigned rc_band_mask(int n_samples, int os, int crop_lo, int crop_hi) {
+    if (!rc_split_supported(n_samples, os) || os < 4 || n_samples > 512 || n_samples * os > 8192) return 0;
+    if (crop_hi / os - crop_lo / os >= 256) return 0;
+    unsigned mask = 0;
+    for (int q = crop_lo / os; q <= crop_hi / os; ++q) mask |= 1u << ((q & 255) >> 4);
+    return mask;
+}
 
 bool rc_split_supported(int n_samples, int os) {
     if (os < 1 || os > 16 || (os & (os - 1)) != 0) return false;
@@ -764,8 +1078,10 @@ bool rc_split_supported(int n_samples, int os) {
 
 cudaError_t launch_range_compress_split(const RcSplitArgs &a, int sign, int mode, cudaStream_t s,
                                         const RcSplitBatch *tab, long long groups) {
-    if (mode == kRcSpectrum || !rc_split_supported(32 * a.N2, a.os)) return cudaErrorInvalidValue;
+    if (!rc_split_supported(32 * a.N2, a.os) || (mode == kRcSpectrum && tab)) return cudaErrorInvalidValue;
     const RcSplitBatch t = tab ? *tab : RcSplitBatch{};
+    if (mode == kRcSpectrum)
+        return sign > 0 ? launch_split<1, kRcSpectrum>(a, t, groups, s) : launch_split<-1, kRcSpectrum>(a, t, groups, s);
     if (sign > 0)
         return mode == kRcProfileF16 ? launch_split<1, kRcProfileF16>(a, t, groups, s)
                                      : launch_split<1, kRcProfileF32>(a, t, groups, s);

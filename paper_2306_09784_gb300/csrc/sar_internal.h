@@ -60,6 +60,11 @@ struct RcSplitArgs {
     long long rows;
     int R, N2, os;
     int crop_lo, crop_hi, n_bins;
+    // band kernel (band != 0: the blocks of 16 values of Q mod 256 it writes)
+    unsigned band;
+    const float4 *pre2;  // [16][threads of a row]: w_r[n] W^(n s) of s, s + 1 (re, re, im, im)
+    const float2 *twd2;  // [16][16]: W_256^(b k1) at [k1][b]
+    const float4 *cmb;   // [N / 256][bin pairs]: W_N^(n2 Q) times the per-bin rotation (re, re, im, im)
 };
 // Batched form: several jobs with the same N, os, convention and storage in
 // one launch; job j owns row groups [group_begin[j], group_begin[j + 1]).
@@ -69,6 +74,8 @@ struct RcSplitBatch {
     int n_jobs;
 };
 bool rc_split_supported(int n_samples, int os);
+unsigned rc_band_mask(int n_samples, int os, int crop_lo, int crop_hi);
+int rc_rows_per_group(const RcSplitArgs &a);
 // tab == null: the single job a; otherwise a gives N2 and os of the table's
 // jobs and groups is the table's total row-group count.
 cudaError_t launch_range_compress_split(const RcSplitArgs &a, int sign, int mode, cudaStream_t s,

@@ -16,6 +16,8 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <mutex>
+#include <vector>
 
 #include "sar_internal.h"
 
@@ -956,6 +958,48 @@ __global__ void __launch_bounds__(kSplitThreads, 2) range_compress_band(RcSplitA
     }
 }
 
+// CTAs of `kern` the current device holds at once with this dynamic shared
+// memory.  Looked up once per (device, kernel, size): the attribute and
+// occupancy queries cost more host time than a launch.  The kernel's shared-
+// memory limit is a process-wide attribute: raised to the device's largest,
+// never lowered.
+cudaError_t resident_ctas(const void *kern, int threads, size_t smem, int *ctas) {
+    struct Entry {
+        const void *kern;
+        size_t smem;
+        int dev, ctas;
+    };
+    static std::mutex mu;
+    static std::vector<Entry> known;  // at most the kernels' sizes times the devices
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Entry &k : known)
+        if (k.kern == kern && k.smem == smem && k.dev == dev) {
+            *ctas = k.ctas;
+            return cudaSuccess;
+        }
+    int sms = 0, optin = 0, occ = 0;
+    cudaFuncAttributes fa;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, kern) != cudaSuccess)
+        return cudaErrorInvalidConfiguration;
+    const int max_dyn = optin - (int)fa.sharedSizeBytes;
+    if ((int)smem > max_dyn) return cudaErrorInvalidValue;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn);
+    if (e != cudaSuccess) return e;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem) != cudaSuccess || occ < 1)
+        return cudaErrorInvalidConfiguration;
+    *ctas = sms * occ;
+    try {
+        known.push_back(Entry{kern, smem, dev, *ctas});
+    } catch (...) {  // not remembered
+    }
+    return cudaSuccess;
+}
+
 template <int SGN, int MODE>
 cudaError_t launch_rc(const RcArgs &a, cudaStream_t s) {
     const int n = a.n_fft;
@@ -971,22 +1015,10 @@ cudaError_t launch_rc(const RcArgs &a, cudaStream_t s) {
                     : n == 2048 ? (os4 ? range_compress_persistent<SGN, MODE, 11, 4>
                                        : range_compress_persistent<SGN, MODE, 11, 16>)
                                 : range_compress_persistent<SGN, MODE, 0, 16>;
-        int dev = 0, sms = 0, optin = 0, occ = 0;
-        cudaFuncAttributes fa;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-            cudaFuncGetAttributes(&fa, kern) != cudaSuccess)
-            return cudaErrorInvalidConfiguration;
-        // process-wide attribute: the largest dynamic size the device allows
-        // next to the kernel's static shared memory
-        const int max_dyn = optin - (int)fa.sharedSizeBytes;
-        if ((int)smem > max_dyn) return cudaErrorInvalidValue;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn);
+        int ctas = 0;
+        const cudaError_t e = resident_ctas((const void *)kern, 256, smem, &ctas);
         if (e != cudaSuccess) return e;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, smem) != cudaSuccess || occ < 1)
-            return cudaErrorInvalidConfiguration;
-        const long long grid = std::min<long long>(n_groups, (long long)sms * occ);
+        const long long grid = std::min<long long>(n_groups, ctas);
         kern<<<(unsigned)grid, 256, smem, s>>>(a, n_groups);
         return cudaGetLastError();
     }
@@ -1041,13 +1073,10 @@ cudaError_t launch_split(const RcSplitArgs &a, const RcSplitBatch &tab, long lon
     rpc = rc_rows_per_group(a);
     long long n_groups = tab.jobs ? groups : (a.rows + rpc - 1) / rpc;
     if (n_groups == 0) return cudaSuccess;
-    int dev = 0, sms = 0, occ = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSplitThreads, smem) != cudaSuccess || occ < 1)
-        return cudaErrorInvalidConfiguration;
-    const long long grid = std::min<long long>(n_groups, (long long)sms * occ);
+    int ctas = 0;
+    const cudaError_t e = resident_ctas(kern, kSplitThreads, smem, &ctas);
+    if (e != cudaSuccess) return e;
+    const long long grid = std::min<long long>(n_groups, ctas);
     RcSplitArgs arg = a;
     RcSplitBatch t = tab;
     void *params[] = {&arg, &t, &n_groups};

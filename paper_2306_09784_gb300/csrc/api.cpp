@@ -682,11 +682,12 @@ size_t profile_bytes(const sar_plan *pl, int M) {
 
 // Workspace of the pair kernel: 16 bytes per bin of max_pulses chirps, twice
 // an FP32 profile buffer.  A plan goes without (and uses the copying kernel)
-// where it would take more than 1 GiB or a sixteenth of the free memory, or
+// where no call of its size takes that path, where it would take more than 1 GiB or a sixteenth of the free memory, or
 // where an HBM budget would then no longer hold the buffers that
 // sar_form_image_host and sar_plan_set_tile_shape allocate later.
 void add_pair_workspace(sar_plan *pl) {
     const size_t rows = (size_t)pl->p.max_pulses * pl->p.n_rx;
+    if ((long long)pl->n_tiles * (long long)rows < kPairMinWindows) return;  // no call is large enough
     const size_t bytes = rows * pl->n_bins * sizeof(float4);
     const size_t geo = rows * sizeof(float4) + (size_t)pl->p.max_pulses * sizeof(float);
     size_t free_b = 0, total_b = 0;

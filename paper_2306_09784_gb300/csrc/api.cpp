@@ -78,7 +78,7 @@ struct sar_plan {
     float2 *d_partial = nullptr;
     int *d_arrived = nullptr;
     int *d_err = nullptr;
-    double *d_means = nullptr;  // sar_doppler_offsets: mean positions and velocity
+    double *d_means = nullptr;  // sar_doppler_offsets: partial sums of positions and velocities
     // tables of the split-transform range compression (when supported)
     bool rc_split = false;
     float2 *d_rc_pre = nullptr, *d_rc_twd = nullptr;
@@ -899,7 +899,7 @@ int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t bud
     }
     if (!rc) {
         void *q = nullptr;
-        rc = dev_alloc(pl, sizeof(double) * 8, &q);
+        rc = dev_alloc(pl, sizeof(double) * 6 * kMeanCtas, &q);
         pl->d_means = (double *)q;
     }
     if (rc) {
@@ -1294,7 +1294,7 @@ int sar_doppler_offsets(sar_plan *pl, const double *q_tx_dev, const double *q_rx
     a.pix = pl->d_pix;
     a.out_idx = pl->d_out;
     a.n_tiles = pl->n_tiles;
-    a.means = pl->d_means;
+    a.sums = pl->d_means;
     // f0 at the transform's time origin (the carrier the phase correction uses)
     const double f0 = pl->beta_frac * pl->p.c * pl->a1;
     a.scale = f0 / pl->p.c * (double)pl->n_fft / pl->p.fs;

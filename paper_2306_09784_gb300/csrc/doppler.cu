@@ -7,8 +7,8 @@
 // the rate of change of the two-way path (a platform closing on p shortens
 // it) times f0 / c, in bins of the range transform.
 //
-// Two kernels: one CTA reduces the means in FP64; then one thread per pixel
-// slot of the plan's tiles (positions = FP64 tile reference + FP32 offset)
+// Two kernels: a few CTAs sum positions and velocities in FP64; then one thread
+// per pixel slot of the plan's tiles (positions = FP64 tile reference + FP32 offset)
 // writes its offset at the pixel's image index.  Both read device memory only
 // (graph-capturable).
 #include "sar_internal.h"
@@ -16,7 +16,10 @@
 namespace sar {
 namespace {
 
-constexpr int kMeanThreads = 1024;
+// Partial sums by kMeanCtas CTAs of 256 threads: one CTA is bound by its SM's
+// two FP64 lanes (the adds and the warp reductions of 1024 chirps x 8 Rx take
+// 15 us there) and by one load in flight.
+constexpr int kMeanThreads = 256;
 
 // (e . v) / |e| with FP64 accuracy far beyond the FP32 result: 1 / |e| from an
 // FP32 reciprocal square root and one Newton step (relative error ~1e-13).  The
@@ -36,17 +39,17 @@ __device__ __forceinline__ double radial(double ex, double ey, double vx, double
     return dot * fma(0.5 * y0, fma(-d2 * y0, y0, 1.0), y0);
 }
 
-// means[0..5] = (qt.x, qt.y, qr.x, qr.y, vbar.x, vbar.y)
-__global__ void __launch_bounds__(kMeanThreads) doppler_means_kernel(const double *__restrict__ q_tx,
-                                                                     const double *__restrict__ q_rx,
-                                                                     const double *__restrict__ vel, int M, int R,
-                                                                     double *__restrict__ means) {
+// sums[cta][0..5]: this CTA's share of the sums of (q_tx.x, q_tx.y, q_rx.x,
+// q_rx.y, vel.x, vel.y).
+__global__ void __launch_bounds__(kMeanThreads) doppler_sums_kernel(const double *__restrict__ q_tx,
+                                                                    const double *__restrict__ q_rx,
+                                                                    const double *__restrict__ vel, int M, int R,
+                                                                    double *__restrict__ sums) {
     __shared__ double part[6][kMeanThreads / 32];
     double s[6] = {0, 0, 0, 0, 0, 0};
-    // 1024 threads with four loads of each array in flight: the sums are bound
-    // by memory latency (1024 chirps x 8 Rx: 16 us with 256 threads, one load)
+    const int first = blockIdx.x * kMeanThreads + threadIdx.x, step = kMeanCtas * kMeanThreads;
 #pragma unroll 4
-    for (int m = threadIdx.x; m < M; m += kMeanThreads) {
+    for (int m = first; m < M; m += step) {
         s[0] += q_tx[2 * m];
         s[1] += q_tx[2 * m + 1];
         s[4] += vel[2 * m];
@@ -54,7 +57,7 @@ __global__ void __launch_bounds__(kMeanThreads) doppler_means_kernel(const doubl
     }
     const long long nr = (long long)M * R;
 #pragma unroll 4
-    for (long long i = threadIdx.x; i < nr; i += kMeanThreads) {
+    for (long long i = first; i < nr; i += step) {
         s[2] += q_rx[2 * i];
         s[3] += q_rx[2 * i + 1];
     }
@@ -69,16 +72,24 @@ __global__ void __launch_bounds__(kMeanThreads) doppler_means_kernel(const doubl
     if (threadIdx.x < 6) {
         double v = 0;
         for (int w = 0; w < kMeanThreads / 32; ++w) v += part[threadIdx.x][w];
-        const int c = threadIdx.x;
-        means[c] = v / ((c == 2 || c == 3) ? (double)nr : (double)M);
+        sums[blockIdx.x * 6 + threadIdx.x] = v;
     }
 }
 
 __global__ void __launch_bounds__(256) doppler_offsets_kernel(const TileInfo *__restrict__ tiles,
                                                                const float2 *__restrict__ pix,
                                                                const int *__restrict__ out_idx, long long slots,
-                                                               const double *__restrict__ means, double scale,
-                                                               float *__restrict__ fd) {
+                                                               const double *__restrict__ sums, int M, long long nr,
+                                                               double scale, float *__restrict__ fd) {
+    __shared__ double means[6];  // (qt.x, qt.y, qr.x, qr.y, vbar.x, vbar.y)
+    if (threadIdx.x < 6) {
+        const int c = threadIdx.x;
+        double v = 0;
+#pragma unroll
+        for (int k = 0; k < kMeanCtas; ++k) v += sums[k * 6 + c];
+        means[c] = v / ((c == 2 || c == 3) ? (double)nr : (double)M);
+    }
+    __syncthreads();
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= slots) return;
     const int o = out_idx[s];
@@ -97,13 +108,13 @@ __global__ void __launch_bounds__(256) doppler_offsets_kernel(const TileInfo *__
 }  // namespace
 
 cudaError_t launch_doppler_offsets(const DopplerArgs &a, cudaStream_t s) {
-    doppler_means_kernel<<<1, kMeanThreads, 0, s>>>(a.q_tx, a.q_rx, a.vel, a.M, a.R, a.means);
+    doppler_sums_kernel<<<kMeanCtas, kMeanThreads, 0, s>>>(a.q_tx, a.q_rx, a.vel, a.M, a.R, a.sums);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const long long slots = (long long)a.n_tiles * kTilePx;
     if (slots == 0) return cudaSuccess;
     doppler_offsets_kernel<<<(unsigned)((slots + 255) / 256), 256, 0, s>>>(a.tiles, a.pix, a.out_idx, slots,
-                                                                            a.means, a.scale, a.fd);
+                                                                            a.sums, a.M, (long long)a.M * a.R, a.scale, a.fd);
     return cudaGetLastError();
 }
 

@@ -223,6 +223,7 @@ cudaError_t launch_backproject_class(const BpClassArgs &c, const BpCheck &chk, s
 cudaError_t launch_batch_fixup(const BpMultiArgs &m, const BpCheck &chk, int total_tiles, cudaStream_t s);
 
 // Per-pixel Doppler offsets (doppler.cu).
+constexpr int kMeanCtas = 16;  // CTAs that sum positions and velocities
 struct DopplerArgs {
     const double *q_tx, *q_rx, *vel;  // [M][2], [M][R][2], [M][2]
     int M, R;
@@ -230,7 +231,7 @@ struct DopplerArgs {
     const float2 *pix;
     const int *out_idx;
     int n_tiles;
-    double *means;  // [6] device scratch of the plan
+    double *sums;  // [kMeanCtas][6] device scratch of the plan
     double scale;   // f0 / c * N_fft / fs: bins per (m/s) of path rate
     float *fd;      // [n_pixels] output in image order
 };

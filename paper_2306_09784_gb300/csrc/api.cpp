@@ -60,12 +60,10 @@ struct sar_plan {
     float4 *d_pairs = nullptr, *d_rx = nullptr, *d_zero = nullptr;
     float *d_o2max = nullptr;
     int zero_len = 0;
-    unsigned long long *d_call = nullptr;
-    unsigned epoch = 0;
-    // the stream and the end of the last call that used the workspace: a call
-    // on another stream waits for it
-    cudaStream_t pair_stream = nullptr;
-    cudaEvent_t pair_done = nullptr;
+    unsigned *d_call = nullptr;
+    // the end of the last backprojection: calls share the plan's pairs,
+    // partial sums and arrival counters, so that one on another stream waits
+    cudaEvent_t bp_done = nullptr;
     size_t pair_smem = 0;
     int pair_G = 0, mb_cap = kMaxPulsesPerBlock;
     // device memory owned by the plan
@@ -245,7 +243,7 @@ void free_plan(sar_plan *pl) {
     cudaDeviceSynchronize();
     for (void *p : pl->allocs) cudaFree(p);
     if (pl->s_copy) cudaStreamDestroy(pl->s_copy);
-    for (cudaEvent_t e : {pl->ev_start, pl->ev_chunk[0], pl->ev_chunk[1], pl->ev_traj, pl->pair_done})
+    for (cudaEvent_t e : {pl->ev_start, pl->ev_chunk[0], pl->ev_chunk[1], pl->ev_traj, pl->bp_done})
         if (e) cudaEventDestroy(e);
     delete pl;
 }
@@ -619,7 +617,9 @@ int install_tiling(sar_plan *pl, const HostTiles &ht, int tw, int L) {
         rc = dev_alloc(pl, sums + counts, &q);
         t.d_partial = (float2 *)q;
         t.d_arrived = (int *)((char *)q + sums);
-        if (!rc && cudaMemset(t.d_arrived, 0, counts) != cudaSuccess) rc = SAR_ECUDA;
+        // (calls may come on streams that do not wait for the memset)
+        if (!rc && (cudaMemset(t.d_arrived, 0, counts) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess))
+            rc = SAR_ECUDA;
     }
     if (rc) return rc;  // what was allocated is freed with the plan
     pl->tilings.push_back(t);
@@ -714,12 +714,12 @@ void add_pair_workspace(sar_plan *pl) {
     void *small = nullptr, *pairs = nullptr;
     if (dev_alloc(pl, rx_o + geo, &small) || dev_alloc(pl, bytes, &pairs) ||
         cudaMemset(small, 0, rx_o) != cudaSuccess ||
-        cudaEventCreateWithFlags(&pl->pair_done, cudaEventDisableTiming) != cudaSuccess) {
+        cudaStreamSynchronize(nullptr) != cudaSuccess) {  // calls may come on streams that do not wait for it
         cudaGetLastError();
         return;
     }
     pl->d_pairs = (float4 *)pairs;
-    pl->d_call = (unsigned long long *)small;
+    pl->d_call = (unsigned *)small;
     pl->d_zero = (float4 *)((char *)small + 256);
     pl->zero_len = zero_len;
     pl->d_rx = (float4 *)((char *)small + rx_o);
@@ -906,6 +906,11 @@ int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t bud
         free_plan(pl);
         return rc;
     }
+    if (cudaEventCreateWithFlags(&pl->bp_done, cudaEventDisableTiming) != cudaSuccess) {
+        pl->bp_done = nullptr;
+        free_plan(pl);
+        return SAR_ECUDA;
+    }
     add_pair_workspace(pl);
     recall_shape(pl);
     *out = pl;
@@ -1089,35 +1094,20 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
     e.rx = pl->d_rx;
     e.o2max = pl->d_o2max;
     e.call = pl->d_call;
-    e.epoch = ++pl->epoch;
     e.rows = a.M * a.R;
     e.R = a.R;
     e.n_bins = a.n_bins;
     e.cb_k = a.cb_k;
     e.inv_kappa = a.inv_kappa;
     const BpLaunch l{pl->rg, pl->fp16, pl->pair_smem, pl->minb};
-    DeviceGuard dg(pl->device);
-    if (!dg.ok) return SAR_ECUDA;
-    // (a captured call is ordered by its graph)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return SAR_ECUDA;
-    if (cap == cudaStreamCaptureStatusNone && s != pl->pair_stream &&
-        cudaStreamWaitEvent(s, pl->pair_done, 0) != cudaSuccess)
-        return SAR_ECUDA;
-    if (launch_backproject_pairs(pa, e, l, s) != cudaSuccess) return SAR_ECUDA;
-    if (cap == cudaStreamCaptureStatusNone) {
-        if (cudaEventRecord(pl->pair_done, s) != cudaSuccess) return SAR_ECUDA;
-        pl->pair_stream = s;
-    }
-    return SAR_OK;
+    // the call's words start from zero here, not by the call's number: a
+    // captured call runs many times
+    if (cudaMemsetAsync(pl->d_call, 0, 16, s) != cudaSuccess) return SAR_ECUDA;
+    return launch_backproject_pairs(pa, e, l, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
-int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const double *q_rx, const float *fd,
-              void *image, int accumulate, cudaStream_t s, int m0 = 0, int M_tot = 0,
-              void *image_out = nullptr) {
-    BpArgs a = common_bp_args(pl, prof, M, q_tx, q_rx, fd, image, accumulate, m0, M_tot);
-    a.image_out = (float2 *)image_out;
-    if (use_pairs(pl, M)) return bp_launch_pairs(pl, a, s);
+// Backprojection of a call's arguments a by the copying kernel.
+int bp_launch_copying(sar_plan *pl, BpArgs a, cudaStream_t s) {
     // a call too small for the pair kernel cuts its pulse blocks so that the
     // CTAs' counts of them even out: the block that minimises, in windows'
     // time, the longest CTA (a block's set-up is worth kBlockSetup windows)
@@ -1126,7 +1116,7 @@ int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const d
         long long best = INT64_MAX;
         int mb = a.Mb;
         for (int b = a.Mb; b >= 1; --b) {
-            const long long per_tile = (M + b - 1) / b, rounds = (a.n_tiles * per_tile + pl->G - 1) / pl->G;
+            const long long per_tile = (a.M + b - 1) / b, rounds = (a.n_tiles * per_tile + pl->G - 1) / pl->G;
             const long long cost = 2 * rounds * ((long long)b * a.R + kBlockSetup) + per_tile;
             if (cost < best) {
                 best = cost;
@@ -1134,14 +1124,31 @@ int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const d
             }
         }
         a.Mb = mb;
-        a.blocks_per_tile = (M + mb - 1) / mb;
+        a.blocks_per_tile = (a.M + mb - 1) / mb;
         a.units = (long long)a.n_tiles * a.blocks_per_tile;
     }
     if (!set_launch(pl, a, pl->d_partial, pl->partial_slots)) return SAR_EINVAL;  // cannot happen
     BpLaunch l{pl->rg, pl->fp16, pl->bp_smem, pl->minb};
+    return launch_backproject(a, l, pl->d_arrived, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
+}
+
+int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const double *q_rx, const float *fd,
+              void *image, int accumulate, cudaStream_t s, int m0 = 0, int M_tot = 0,
+              void *image_out = nullptr) {
+    BpArgs a = common_bp_args(pl, prof, M, q_tx, q_rx, fd, image, accumulate, m0, M_tot);
+    a.image_out = (float2 *)image_out;
     DeviceGuard dg(pl->device);
     if (!dg.ok) return SAR_ECUDA;
-    return launch_backproject(a, l, pl->d_arrived, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
+    // order after the last call, whichever stream that ran on: handles do not
+    // tell streams apart (reuse, per-thread default streams), and on the same
+    // stream the wait is free (a captured call is ordered by its graph)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return SAR_ECUDA;
+    const bool live = cap == cudaStreamCaptureStatusNone;
+    if (live && cudaStreamWaitEvent(s, pl->bp_done, 0) != cudaSuccess) return SAR_ECUDA;
+    const int rc = use_pairs(pl, M) ? bp_launch_pairs(pl, a, s) : bp_launch_copying(pl, a, s);
+    if (rc) return rc;
+    return !live || cudaEventRecord(pl->bp_done, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
 }  // namespace

@@ -7,8 +7,9 @@
 //  * Persistent grid of (SMs x resident CTAs).  The work units (pixel tile,
 //    pulse block) are split into equal contiguous ranges, one per CTA
 //    ("stream-K"): every CTA does the same number of pulse blocks.  A tile
-//    split across CTAs is summed by bp_fixup_kernel in CTA order, so results
-//    are deterministic for a given grid.
+//    split across CTAs is summed in CTA order by the last warp to arrive, or
+//    by bp_fixup_kernel where there are no arrival counters, so results are
+//    deterministic for a given grid.
 //  * Each thread keeps 4 pixels in registers: offsets (dx, dy) from the tile
 //    reference point and the complex accumulators.
 //  * Per (tile, pulse, antenna) the reference range R0 to the tile reference

@@ -14,9 +14,9 @@
 //    16-byte entries were 1-2 % slower on frames and 15 % on point lists.
 //  * What bounds it: the packed FMA, MUFU and shared-memory pipes at 57-62 %
 //    each of the time and instruction issue at 61 %, as in backproject.cu.
-//    512 x 512 x 1024 x 4 FP32 frame: 0.85 -> 0.78 ms; 1024 x 1024 x 2048 x 4
-//    FP16: 6.42 -> 6.07 ms; 165 000 polar points x 1024 x 8 with Doppler
-//    offsets: 6.07 -> 2.44 ms.
+//    With the expansion, against the copying kernel: 512 x 512 x 1024 x 4 FP32
+//    frame 0.86 -> 0.79 ms; 1024 x 1024 x 2048 x 4 FP16 6.42 -> 6.10 ms;
+//    165 000 polar points x 1024 x 8 with Doppler offsets 6.07 -> 2.44 ms.
 //  * The window is cut to the bins the tile can reach: its own radius and the
 //    call's largest Rx offset (reduced by the expansion kernel) instead of
 //    the plan-wide length, which a point list's widest run of 1024 points
@@ -96,7 +96,7 @@ __device__ __forceinline__ PairLayout pair_layout(const BpPairArgs &pa, const Ti
     const BpArgs &a = pa.b;
     PairLayout l;
     const float a1 = a.a1f, rho = (float)ti.rho;
-    const float omax = __uint_as_float((unsigned)pa.call[0]);
+    const float omax = __uint_as_float(pa.call[0]);
     const float o = fminf(omax, ti.o_allow);
     // reachable indices: [a1 (o_allow - o) + G, a1 (o_allow + o) + 4 a1 rho
     // + 2 fd_max + G + 1] in the expansion loop (window start at klo_off),
@@ -478,7 +478,7 @@ __device__ __forceinline__ bool pair_segment(const BpPairArgs &pa, PairSmem &sm,
         acc_im[j] = 0.f;
     }
     sm.l = pair_layout(pa, ti, m_end - m_begin, pulse_unroll<RG, MULTI>());
-    const bool axis = !(unsigned)pa.call[1];
+    const bool axis = !pa.call[1];
     const int Mt = sm.l.Mt, slots = sm.l.slots;
     const int nb = (m_end - m_begin + Mt - 1) / Mt;
     auto start = [&](int b) { return m_begin + b * Mt; };
@@ -656,8 +656,8 @@ __global__ void __launch_bounds__(kBpThreads, MINB)
 // beta) - S_k) / kappa (see convert_block in backproject.cu); one warp per
 // row, 16 bytes written per bin.  The warp of a pulse's first row also takes
 // the pulse's Rx offsets o = q_rx - q_tx (FP64 differences, FP32 values), their
-// largest square, and into call[0], call[1] the call's largest |o| and whether
-// any o has a y component, under the call's number so that no reset is needed.
+// largest square, and into call[0], call[1] (zero before the launch) the FP32
+// bits of the call's largest |o| and whether any o has a y component.
 template <bool FP16>
 __global__ void __launch_bounds__(256) expand_pairs_kernel(ExpandArgs e) {
     __shared__ unsigned call_sh[2];
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(256) expand_pairs_kernel(ExpandArgs e) {
         }
     }
     __syncthreads();
-    if (threadIdx.x < 2) atomicMax(e.call + threadIdx.x, ((unsigned long long)e.epoch << 32) | call_sh[threadIdx.x]);
+    if (threadIdx.x < 2) atomicMax(e.call + threadIdx.x, call_sh[threadIdx.x]);
 }
 
 template <int RG, bool MULTI>

@@ -187,7 +187,7 @@ struct BpPairArgs {
     const float4 *zero;        // L zero entries
     const float4 *rx;          // [M R] Rx offset (o_x, o_y, |o|^2, 0)
     const float *o2max;        // [M] largest |o|^2 of the pulse
-    const unsigned long long *call;  // low words: FP32 bits of the call's largest |o|; any o_y
+    const unsigned *call;      // FP32 bits of the call's largest |o|; any o_y
     int *arrived;              // [n_tiles][8] warps done with a split tile's pixels, zero between launches
     unsigned smem_bytes;       // dynamic shared memory of the launch
     int mb_cap;                // chirps per pipeline block at most
@@ -199,8 +199,7 @@ struct ExpandArgs {
     float4 *pairs;
     float4 *rx;
     float *o2max;
-    unsigned long long *call;
-    unsigned epoch;            // the plan's call number
+    unsigned *call;
     int rows, R, n_bins;
     float2 cb_k;
     float inv_kappa;

@@ -103,3 +103,24 @@ def test_launch_shapes_and_streams():
     for rg, minb, mb in ((4, 3, 5), (2, 2, 7), (1, 2, 1), (4, 2, 1)):
         plan.set_launch(rg, minb, mb)
         _compare(plan, prof, 260, qt, qr)
+
+
+def test_captured_call_replays_with_new_geometry():
+    """A captured call keeps no result of other calls: replayed after a call with
+    a much smaller array and with its own array widened in place, it still
+    stages every bin that its geometry reaches."""
+    import torch
+    M = 260
+    plan, prof, qt, qr, _ = _frames(4, M, synth.Grid(-4.1, 1.2, 0.033, 0.03, 250, 270))
+    img = torch.zeros(plan.n_pixels, dtype=torch.complex64, device="cuda")
+    plan.backproject(prof, M, qt, qr, image=img)  # modules loaded before the capture
+    torch.cuda.synchronize()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        plan.backproject(prof, M, qt, qr, image=img, stream=s)
+    small = (qt[:, None, :] + 0.02 * (qr - qt[:, None, :])).contiguous()
+    _compare(plan, prof, M, qt, small)
+    qr.copy_(qt[:, None, :] + 6.0 * (qr - qt[:, None, :]))
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(img, _compare(plan, prof, M, qt, qr))

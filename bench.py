@@ -50,16 +50,17 @@ MUFU_LANES = 16
 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one
-# backprojection launch on this workload, from an ncu capture of the kernel
-# source with this SHA-256 prefix (reported as null once the kernel source
-# differs).
-BP_TRAFFIC = {"sha256_16": "c349ed253e1a87fd", "bytes": 32666112 + 4608}
+# backprojection call on this workload (the expansion's and the pair kernel's
+# launch), from an ncu capture of the kernel source with this SHA-256 prefix
+# (reported as null once the kernel source differs).
+BP_TRAFFIC = {"sha256_16": "805b979ef1256bae",
+              "bytes": 21308416 + 23238144 + 149230336 + 5760000}
 HBM_PEAK_FALLBACK_GBS = 6800.0
 
 
 def kernel_traffic():
     import hashlib
-    src = os.path.join(ROOT, "paper_2306_09784_gb300", "csrc", "backproject.cu")
+    src = os.path.join(ROOT, "paper_2306_09784_gb300", "csrc", "backproject_pairs.cu")
     try:
         h = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
     except OSError:
@@ -736,7 +737,7 @@ def run_ours(args):
                        "range_compress_mean": statistics.mean(rc_ms),
                        "backproject_mean": statistics.mean(bp_ms)},
         "per_chirp_rate": value / R,
-        "roofline": {"bound": "alu", "kernel": "backproject_kernel (+ fix-up)",
+        "roofline": {"bound": "alu", "kernel": "backproject_pairs_kernel (+ expand_pairs_kernel)",
                      "achieved": achieved, "peak": peak, "unit": "Gupdate/s",
                      "frac": achieved / peak, "traffic": kernel_traffic(),
                      "peak_basis": "min(152 SM x 128 FP32 lanes / 17 ops, 152 SM x 16 MUFU "

@@ -15,7 +15,7 @@
 //  * What bounds it: the packed FMA, MUFU and shared-memory pipes at 57-62 %
 //    each of the time and instruction issue at 61 %, as in backproject.cu.
 //    With the expansion, against the copying kernel: 512 x 512 x 1024 x 4 FP32
-//    frame 0.86 -> 0.79 ms; 1024 x 1024 x 2048 x 4 FP16 6.42 -> 6.10 ms;
+//    frame 0.86 -> 0.79 ms; 1024 x 1024 x 2048 x 4 FP16 6.42 -> 6.14 ms;
 //    165 000 polar points x 1024 x 8 with Doppler offsets 6.07 -> 2.44 ms.
 //  * The window is cut to the bins the tile can reach: its own radius and the
 //    call's largest Rx offset (reduced by the expansion kernel) instead of

@@ -259,9 +259,10 @@ int sar_range_spectrum(sar_plan *plan, const void *beat_dev, int32_t M,
  * interpolation index would leave the staged bin window.
  * Large calls go through a workspace of the plan that holds the profiles as
  * interpolation pairs (16 bytes per bin of max_pulses chirps, part of
- * device_bytes; a plan goes without it where it would take over 1 GiB or a
+ * device_bytes; sar_plan_pair_path tells which calls).  A plan goes without it
+ * where no call of its sizes would gain, where it would take over 1 GiB or a
  * sixteenth of the free memory, or where its HBM budget would not hold the
- * buffers allocated later).  A call on another stream than the previous one
+ * buffers allocated later.  A call on another stream than the previous one
  * waits for it.
  */
 int sar_backproject(sar_plan *plan, const void *prof_dev, int32_t M,
@@ -582,6 +583,14 @@ int sar_plan_set_launch(sar_plan *plan, int32_t rx_group, int32_t regs_ctas_per_
  * plan.
  */
 int sar_plan_set_tile_shape(sar_plan *plan, int32_t tile_w);
+
+/*
+ * Whether sar_backproject calls of M chirps go through the plan's pair
+ * workspace (*taken = 1; see sar_backproject) with the plan's current tile
+ * shape, and the workspace's size in device memory (0: the plan has none;
+ * workspace_bytes may be NULL).
+ */
+int sar_plan_pair_path(const sar_plan *plan, int32_t M, int32_t *taken, size_t *workspace_bytes);
 
 /*
  * Waits for the plan's device work and reports (then clears) kernel-side

@@ -33,7 +33,7 @@ EXPORTS = (
     "sar_release", "sar_server_get_stats", "sar_plan_autotune", "sar_plan_set_launch",
     "sar_alu_peaks", "sar_polar_grid", "sar_doppler_offsets", "sar_batch_autotune",
     "sar_batch_num_classes", "sar_batch_get_class", "sar_batch_check_errors", "sar_batch_add_frame",
-    "sar_plan_set_tile_shape",
+    "sar_plan_set_tile_shape", "sar_plan_pair_path",
 )
 REQ_QUEUED, REQ_RUNNING, REQ_DONE, REQ_FAILED = range(4)
 
@@ -164,6 +164,7 @@ def load_library(path: str = LIB_PATH):
     lib.sar_batch_check_errors.argtypes = [vp, ctypes.POINTER(i32)]
     lib.sar_batch_add_frame.argtypes = [vp, vp, vp, vp, vp, i32, vp, vp, vp, i32]
     lib.sar_plan_set_tile_shape.argtypes = [vp, i32]
+    lib.sar_plan_pair_path.argtypes = [vp, i32, ctypes.POINTER(i32), ctypes.POINTER(sz)]
     for name in EXPORTS:
         fn = getattr(lib, name)
         if name not in ("sar_plan_destroy", "sar_status_string", "sar_batch_destroy",
@@ -399,6 +400,14 @@ class Plan:
         _check(self._lib.sar_plan_set_launch(self._plan, rx_group, regs_ctas_per_sm,
                                              pulses_per_block), "sar_plan_set_launch")
         return self.launch_shape()
+
+    def pair_path(self, M: int) -> tuple:
+        """(whether backproject calls of M chirps go through the pair
+        workspace, its size in bytes; see sar_plan_pair_path)."""
+        taken, n = ctypes.c_int32(), ctypes.c_size_t()
+        _check(self._lib.sar_plan_pair_path(self._plan, M, ctypes.byref(taken), ctypes.byref(n)),
+               "sar_plan_pair_path")
+        return bool(taken.value), int(n.value)
 
     def check_errors(self) -> int:
         return self._lib.sar_plan_check_errors(self._plan)

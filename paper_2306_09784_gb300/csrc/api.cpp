@@ -27,11 +27,10 @@ constexpr int kMaxPulsesPerBlock = 32;
 constexpr size_t kPairSmem[2] = {113 * 1024, 75 * 1024};
 // Largest workspace of interpolation pairs a plan keeps.
 constexpr size_t kPairBytesMax = size_t(1) << 30;
-// Calls of at least this many windows (pixel tiles x chirps x Rx, 6.7e7 updates,
-// ~50 us) take the pair kernel.  Its extra launch and the pairs it writes cost
-// ~5 us, its pixel loop saves ~8 %: 131072 windows in 139 us against 144 us,
-// 4096 windows in 32 us against 29 us.
-constexpr long long kPairMinWindows = 65536;
+// GPU time (ps) that the pair kernel saves per window (pixel tile x chirp x Rx)
+// of L bins, and spends, against the copying kernel (see pairs_pay).
+constexpr double kPairPerWindow = 52.0, kPairPerWindowBin = 3.8, kPairPerPulseTile = 365.0;
+constexpr double kPairPerCall = 12.0e6, kPairPerTile = 3.5e3, kPairPerRowBin = 7.4;
 // Set-up of a pulse block of the copying kernel, in windows' time (~1 us, 12 of
 // ~70 ns): 128 x 128 x 256 x 1 frame 24.6 us at blocks of 16 or 32 chirps, 28.7
 // at 24, where the last CTAs of a second round run alone.
@@ -64,7 +63,7 @@ struct sar_plan {
     // the end of the last backprojection: calls share the plan's pairs,
     // partial sums and arrival counters, so that one on another stream waits
     cudaEvent_t bp_done = nullptr;
-    size_t pair_smem = 0;
+    size_t pair_smem = 0, pair_bytes = 0;
     int pair_G = 0, mb_cap = kMaxPulsesPerBlock;
     // device memory owned by the plan
     float *d_wr = nullptr;
@@ -680,14 +679,34 @@ size_t profile_bytes(const sar_plan *pl, int M) {
     return rows * pl->n_bins * 8;
 }
 
+// Whether the pair kernel is the faster one for calls of M chirps (the current
+// tiling).  Against the copying kernel it saves the conversion of every window's
+// bins and some set-up per (window, Rx), and it spends an expansion of whole
+// profile rows, reach word and launch per call, set-up per tile, and more per
+// (tile, chirp) than a single Rx gives back.  The six figures are a fit to 400
+// calls timed on both kernels (24 to 2600 pixels a side, 1 to 4096 chirps, 1 to
+// 16 Rx, 38 to 4096 bins, windows of 20 to 132): the rule's choice is 0.3 %
+// slower than the faster kernel on average, and at worst 5 % slower than the
+// copying kernel.  1024 chirps x 4 Rx on 256 tiles: 817 us against 884; 64 x 64
+// pixels, 16384 chirps of 2048 bins each: 279 us against 99, not taken; 2048 x
+// 2048 pixels, 16 chirps: 154 against 107, not taken; one Rx, windows of 20
+// bins, 2298 chirps on 275 tiles: 757 against 733, not taken.
+bool pairs_pay(const sar_plan *pl, int M) {
+    const double rows = (double)M * pl->p.n_rx, windows = rows * pl->n_tiles;
+    const double saved = windows * (kPairPerWindow + kPairPerWindowBin * pl->L - kPairPerPulseTile / pl->p.n_rx);
+    return saved > kPairPerCall + kPairPerTile * pl->n_tiles + kPairPerRowBin * rows * pl->n_bins;
+}
+
 // Workspace of the pair kernel: 16 bytes per bin of max_pulses chirps, twice
 // an FP32 profile buffer.  A plan goes without (and uses the copying kernel)
-// where no call of its size takes that path, where it would take more than 1 GiB or a sixteenth of the free memory, or
-// where an HBM budget would then no longer hold the buffers that
-// sar_form_image_host and sar_plan_set_tile_shape allocate later.
+// where no call of its size takes that path (what a call saves less what it
+// spends grows with its chirps), where it would take more than 1 GiB or a
+// sixteenth of the free memory, or where an HBM budget would then no longer
+// hold the buffers that sar_form_image_host and sar_plan_set_tile_shape
+// allocate later.
 void add_pair_workspace(sar_plan *pl) {
     const size_t rows = (size_t)pl->p.max_pulses * pl->p.n_rx;
-    if ((long long)pl->n_tiles * (long long)rows < kPairMinWindows) return;  // no call is large enough
+    if (!pairs_pay(pl, pl->p.max_pulses)) return;
     const size_t bytes = rows * pl->n_bins * sizeof(float4);
     const size_t geo = rows * sizeof(float4) + (size_t)pl->p.max_pulses * sizeof(float);
     size_t free_b = 0, total_b = 0;
@@ -719,12 +738,16 @@ void add_pair_workspace(sar_plan *pl) {
         return;
     }
     pl->d_pairs = (float4 *)pairs;
+    pl->pair_bytes = bytes + rx_o + geo;
     pl->d_call = (unsigned *)small;
     pl->d_zero = (float4 *)((char *)small + 256);
     pl->zero_len = zero_len;
     pl->d_rx = (float4 *)((char *)small + rx_o);
     pl->d_o2max = (float *)(pl->d_rx + rows);
-    if (!pair_launch(pl, pl->rg, pl->minb, &pl->pair_smem, &pl->pair_G)) pl->d_pairs = nullptr;
+    if (!pair_launch(pl, pl->rg, pl->minb, &pl->pair_smem, &pl->pair_G)) {
+        pl->d_pairs = nullptr;
+        pl->pair_bytes = 0;
+    }
 }
 
 int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t budget, sar_plan **out) {
@@ -1061,8 +1084,7 @@ bool set_launch(const sar_plan *pl, BpArgs &a, float2 *partial, size_t slots) {
 }
 
 bool use_pairs(const sar_plan *pl, int M) {
-    return pl->d_pairs && pl->L <= pl->zero_len &&
-           (long long)pl->n_tiles * M * pl->p.n_rx >= kPairMinWindows;
+    return pl->d_pairs && pl->L <= pl->zero_len && pairs_pay(pl, M);
 }
 
 // Backprojection from interpolation pairs of a call's arguments a.
@@ -2047,6 +2069,13 @@ int sar_plan_set_tile_shape(sar_plan *pl, int32_t tile_w) {
     } catch (const std::bad_alloc &) {
         return SAR_ENOMEM;
     }
+}
+
+int sar_plan_pair_path(const sar_plan *pl, int32_t M, int32_t *taken, size_t *workspace_bytes) {
+    if (!pl || !taken || M < 1 || M > pl->p.max_pulses) return SAR_EINVAL;
+    *taken = use_pairs(pl, M) ? 1 : 0;
+    if (workspace_bytes) *workspace_bytes = pl->pair_bytes;
+    return SAR_OK;
 }
 
 int sar_plan_check_errors(sar_plan *pl) {

@@ -593,8 +593,21 @@ int sar_plan_set_tile_shape(sar_plan *plan, int32_t tile_w);
 int sar_plan_pair_path(const sar_plan *plan, int32_t M, int32_t *taken, size_t *workspace_bytes);
 
 /*
+ * Limit of the waits inside the kernels of later sar_backproject calls, in
+ * polls (-1: the default, 2^20, far beyond any copy's time).  Kernels wait
+ * for their own copies from device memory only.  A call whose wait runs out
+ * waits for those copies to land, leaves the rest of its image unwritten and is
+ * reported by sar_plan_check_errors as SAR_ETIMEOUT; 0 gives up at once (to
+ * try the error path).  SAR_EINVAL below -1.
+ */
+int sar_plan_set_wait_limit(sar_plan *plan, int32_t polls);
+
+/*
  * Waits for the plan's device work and reports (then clears) kernel-side
- * error flags: SAR_OK or SAR_EBOUNDS.
+ * error flags of all calls since the last check: SAR_OK, SAR_EBOUNDS (invalid
+ * geometry or offsets were left out) or SAR_ETIMEOUT (a wait inside a kernel
+ * ran out: the image of some call, sar_form_image_host included, is
+ * incomplete).
  */
 int sar_plan_check_errors(sar_plan *plan);
 

@@ -64,6 +64,7 @@ struct sar_plan {
     // partial sums and arrival counters, so that one on another stream waits
     cudaEvent_t bp_done = nullptr;
     size_t pair_smem = 0, pair_bytes = 0;
+    int polls = kWaitPolls;  // of the pair kernel's waits for its copies
     int pair_G = 0, mb_cap = kMaxPulsesPerBlock;
     // device memory owned by the plan
     float *d_wr = nullptr;
@@ -1107,6 +1108,7 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
     pa.div_blk = ((1ull << 32) + (unsigned)a.Mb - 1) / (unsigned)a.Mb;
     pa.smem_bytes = (unsigned)pl->pair_smem;
     pa.mb_cap = pl->mb_cap;
+    pa.polls = pl->polls;
     ExpandArgs e{};
     e.prof = a.prof;
     e.scales = a.prof_scale;
@@ -2078,6 +2080,12 @@ int sar_plan_pair_path(const sar_plan *pl, int32_t M, int32_t *taken, size_t *wo
     return SAR_OK;
 }
 
+int sar_plan_set_wait_limit(sar_plan *pl, int32_t polls) {
+    if (!pl || polls < -1) return SAR_EINVAL;
+    pl->polls = polls < 0 ? kWaitPolls : polls;
+    return SAR_OK;
+}
+
 int sar_plan_check_errors(sar_plan *pl) {
     if (!pl) return SAR_EINVAL;
     DeviceGuard dg(pl->device);
@@ -2088,7 +2096,7 @@ int sar_plan_check_errors(sar_plan *pl) {
     if (h[0] & kErrStall)  // a launch gave up: arrivals of its split tiles are void
         for (const sar_plan::Tiling &t : pl->tilings)
             if (cudaMemset(t.d_arrived, 0, (size_t)t.n_tiles * 8 * sizeof(int)) != cudaSuccess) return SAR_ECUDA;
-    return h[0] ? SAR_EBOUNDS : SAR_OK;
+    return (h[0] & kErrStall) ? SAR_ETIMEOUT : h[0] ? SAR_EBOUNDS : SAR_OK;
 }
 
 }  // extern "C"

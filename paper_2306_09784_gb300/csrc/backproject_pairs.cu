@@ -44,7 +44,7 @@ namespace sar {
 namespace {
 
 // Full barriers of the two table slots, exact-loop bits of the three Tx slots,
-// stall flag.
+// stall bits.
 constexpr unsigned kHeaderBytes = 32;
 constexpr int kWarps = kBpThreads / 32;
 // Slack (bins) on both ends of a staged window: the FP32 index differs from
@@ -69,9 +69,9 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 // Bounded wait of a whole warp (its lanes stay together): false if the phase
-// has not completed after a number of polls that takes far longer than any copy.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    for (int i = 0; i < (1 << 20); ++i)
+// has not completed after `polls` polls.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int polls) {
+    for (int i = 0; i < polls; ++i)
         if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
     return false;
 }
@@ -142,6 +142,8 @@ struct PairSmem {
     __device__ int2 *rxb(int t, int R) const { return reinterpret_cast<int2 *>(base + l.rxb) + t * l.Mt * R; }
     // per Tx slot: bit j set where run j of the block takes the exact loop
     __device__ unsigned *exact(int s) const { return reinterpret_cast<unsigned *>(base) + 4 + s; }
+    // bit b & 1 set: a wait of block b ran out (two bits, so that a warp already
+    // in the next block cannot change what the others read of this one)
     __device__ volatile int *stall() const { return reinterpret_cast<volatile int *>(base) + 7; }
     __device__ uint32_t bar(int t) const { return addr + 8u * t; }
     // first byte of window w of table slot t
@@ -514,8 +516,8 @@ __device__ __forceinline__ bool pair_segment(const BpPairArgs &pa, PairSmem &sm,
                 stage_windows<MULTI, RG>(pa, sm, start(b + 1), count(b + 1), s1, t1, rt1, x_next);
             }
         }
-        if (!mbar_wait(sm.bar(t), (phase >> t) & 1u)) {
-            *sm.stall() = 1;
+        if (!mbar_wait(sm.bar(t), (phase >> t) & 1u, pa.polls)) {
+            *sm.stall() = 1 << (b & 1);
             atomicOr(a.err, kErrStall);
         }
         phase ^= 1u << t;
@@ -538,10 +540,12 @@ __device__ __forceinline__ bool pair_segment(const BpPairArgs &pa, PairSmem &sm,
         }
         if (threadIdx.x == 0) *sm.exact(s) = 0;  // free for block b + 3
         __syncthreads();
-        if (*sm.stall()) {
-            // a copy that never completed: wait (bounded) for what is in
-            // flight before the CTA's shared memory goes away
-            if (more && slots == 2) mbar_wait(sm.bar(t1), (phase >> t1) & 1u);
+        if ((*sm.stall() >> (b & 1)) & 1) {
+            // the call gives up and is flagged; this CTA's remaining work is
+            // left out.  Its copies in flight write into its shared memory, so
+            // they are waited for (bounded) before it goes away.
+            mbar_wait(sm.bar(t), ((phase >> t) & 1u) ^ 1u, kWaitPolls);
+            if (more && slots == 2) mbar_wait(sm.bar(t1), (phase >> t1) & 1u, kWaitPolls);
             return false;
         }
         if (slots == 1 && more) stage_windows<MULTI, RG>(pa, sm, start(b + 1), count(b + 1), s1, t1, rt1, x_next);
@@ -633,7 +637,7 @@ __global__ void __launch_bounds__(kBpThreads, MINB)
         mbar_init(sm.bar(1));
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (threadIdx.x < 4) reinterpret_cast<int *>(smem_bpp)[4 + threadIdx.x] = 0;  // exact-loop bits, stall flag
+    if (threadIdx.x < 4) reinterpret_cast<int *>(smem_bpp)[4 + threadIdx.x] = 0;  // exact-loop bits, stall bits
     __syncthreads();
     uint32_t phase = 0;
     const long long u0 = (long long)blockIdx.x * a.units / a.G;

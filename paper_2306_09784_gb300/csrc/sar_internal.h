@@ -18,10 +18,10 @@ constexpr int kPxPerThread = kTilePx / kBpThreads;
 constexpr int kGuardBins = 2;
 // Absolute distances beyond this (m) are treated as invalid geometry.
 constexpr double kMaxRange = 1.0e6;
-// Bits of the device error flag (any bit set: SAR_EBOUNDS).
+// Bits of the device error flag (SAR_EBOUNDS unless noted).
 constexpr int kErrGeometry = 1;      // non-finite or out-of-range antenna geometry
 constexpr int kErrDopplerBound = 2;  // |f_doppler(p)| beyond the plan's bound, or not finite
-constexpr int kErrStall = 4;         // a bounded wait of a kernel ran out (never expected)
+constexpr int kErrStall = 4;         // a bounded wait of a kernel ran out (SAR_ETIMEOUT)
 
 // Range compression output modes.
 enum RcMode { kRcProfileF32 = 0, kRcProfileF16 = 1, kRcSpectrum = 2 };
@@ -179,6 +179,7 @@ struct BpLaunch {
 
 // Backprojection from interpolation pairs (backproject_pairs.cu).
 constexpr int kPairUnit = 2;  // pulses per work unit
+constexpr int kWaitPolls = 1 << 20;  // polls of a wait for a copy: far longer than any takes
 struct BpPairArgs {
     BpArgs b;                  // units, blocks_per_tile: in units of kPairUnit pulses; Mb: pulses per
                                // aligned run that shares the loop choice; prof unused
@@ -191,6 +192,7 @@ struct BpPairArgs {
     int *arrived;              // [n_tiles][8] warps done with a split tile's pixels, zero between launches
     unsigned smem_bytes;       // dynamic shared memory of the launch
     int mb_cap;                // chirps per pipeline block at most
+    int polls;                 // polls of a copy's barrier before the call gives up
 };
 struct ExpandArgs {
     const void *prof;          // profile samples (float2 or half2)

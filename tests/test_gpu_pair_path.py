@@ -53,3 +53,43 @@ def test_long_windows(n_rx, M, fd, taken):
                                         fd=fd)
     assert plan.pair_path(M)[0] == taken
     _compare(plan, prof, M, qt, qr, fdopp)
+
+
+@pytest.mark.parametrize("case", [
+    dict(heading=0.4), dict(y0=0.1), dict(fd=3.0), dict(fd=3.0, heading=-0.3), dict(sign=-1), dict(crop=(40, 90)),
+    dict(crop=(0, 1023)), dict(os_factor=1), dict(os_factor=16), dict(near=True), dict(precision=1, near=True, fd=2.0)])
+@pytest.mark.parametrize("n_rx,M", [(4, 2201), (6, 701)])
+def test_options(case, n_rx, M):
+    """The options of tests/test_gpu_pairs.py at sizes beyond the line."""
+    case = dict(case)
+    y0 = case.pop("y0", 1.2)
+    if case.pop("near", False):
+        y0 = -3.0
+    plan, prof, qt, qr, fd = _frames(n_rx, M, synth.Grid(-4.1, y0, 0.033, 0.03, 250, 270), **case)
+    assert plan.pair_path(M)[0]
+    _compare(plan, prof, M, qt, qr, fd)
+    _compare(plan, prof, M, qt, qr, fd, accumulate=True)
+
+
+def test_wait_that_runs_out_is_reported():
+    """With no polls every CTA gives up at its first block: the call is flagged
+    as timed out, and after the check the next call is right bit for bit."""
+    import torch
+    import paper_2306_09784_gb300 as sar
+    M = 600
+    plan, prof, qt, qr, _ = _frames(4, M, synth.Grid(-4.1, 1.2, 0.033, 0.03, 250, 270))
+    assert plan.pair_path(M)[0]
+    ref = plan.backproject(prof, M, qt, qr)
+    assert plan.check_errors() == sar.SAR_OK
+    for polls in (-2, -100):
+        with pytest.raises(sar.SarError):
+            plan.set_wait_limit(polls)
+    plan.set_wait_limit(0)
+    left = torch.full_like(ref, complex(7.0, -7.0))
+    plan.backproject(prof, M, qt, qr, image=left)
+    assert plan.check_errors() == sar.SAR_ETIMEOUT
+    assert bool((left == complex(7.0, -7.0)).all())  # nothing half-done was written
+    plan.set_wait_limit()
+    got = plan.backproject(prof, M, qt, qr)
+    assert plan.check_errors() == sar.SAR_OK
+    assert torch.equal(got, ref)

@@ -74,7 +74,8 @@ struct sar_plan {
     int *d_out = nullptr;
     TileInfo *d_tiles = nullptr;
     float2 *d_partial = nullptr;
-    int *d_arrived = nullptr;
+    unsigned long long *d_arrived = nullptr;
+    unsigned long long bp_calls = 0;  // numbered backprojections (see bp_launch_copying)
     int *d_err = nullptr;
     double *d_means = nullptr;  // sar_doppler_offsets: partial sums of positions and velocities
     // tables of the split-transform range compression (when supported)
@@ -107,7 +108,7 @@ struct sar_plan {
         int *d_out = nullptr;
         TileInfo *d_tiles = nullptr;
         float2 *d_partial = nullptr;
-        int *d_arrived = nullptr;  // pair kernel: arrivals of split tiles (after the partial sums)
+        unsigned long long *d_arrived = nullptr;  // arrivals at split tiles (after the partial sums)
     };
     std::vector<Tiling> tilings;
     int tile_w = 0;
@@ -613,10 +614,10 @@ int install_tiling(sar_plan *pl, const HostTiles &ht, int tw, int L) {
     if (!rc) rc = upload(pl, ht.tiles, &t.d_tiles);
     if (!rc) {
         void *q = nullptr;
-        const size_t sums = t.partial_slots * kTilePx * sizeof(float2), counts = (size_t)t.n_tiles * 8 * sizeof(int);
+        const size_t sums = t.partial_slots * kTilePx * sizeof(float2), counts = (size_t)t.n_tiles * 8 * sizeof(unsigned long long);
         rc = dev_alloc(pl, sums + counts, &q);
         t.d_partial = (float2 *)q;
-        t.d_arrived = (int *)((char *)q + sums);
+        t.d_arrived = (unsigned long long *)((char *)q + sums);
         // (calls may come on streams that do not wait for the memset)
         if (!rc && (cudaMemset(t.d_arrived, 0, counts) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess))
             rc = SAR_ECUDA;
@@ -1104,7 +1105,7 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
     pa.rx = pl->d_rx;
     pa.o2max = pl->d_o2max;
     pa.call = pl->d_call;
-    pa.arrived = pl->d_arrived;
+    pa.arrived = BpArrivals{pl->d_arrived, 0};
     pa.div_blk = ((1ull << 32) + (unsigned)a.Mb - 1) / (unsigned)a.Mb;
     pa.smem_bytes = (unsigned)pl->pair_smem;
     pa.mb_cap = pl->mb_cap;
@@ -1118,6 +1119,8 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
     e.rx = pl->d_rx;
     e.o2max = pl->d_o2max;
     e.call = pl->d_call;
+    e.arrived = pl->d_arrived;
+    e.n_arrived = a.n_tiles * 8;
     e.rows = a.M * a.R;
     e.R = a.R;
     e.n_bins = a.n_bins;
@@ -1130,8 +1133,9 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
     return launch_backproject_pairs(pa, e, l, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
-// Backprojection of a call's arguments a by the copying kernel.
-int bp_launch_copying(sar_plan *pl, BpArgs a, cudaStream_t s) {
+// Backprojection of a call's arguments a by the copying kernel.  live: enqueued
+// now, not captured.
+int bp_launch_copying(sar_plan *pl, BpArgs a, cudaStream_t s, bool live) {
     // a call too small for the pair kernel cuts its pulse blocks so that the
     // CTAs' counts of them even out: the block that minimises, in windows'
     // time, the longest CTA (a block's set-up is worth kBlockSetup windows)
@@ -1153,7 +1157,15 @@ int bp_launch_copying(sar_plan *pl, BpArgs a, cudaStream_t s) {
     }
     if (!set_launch(pl, a, pl->d_partial, pl->partial_slots)) return SAR_EINVAL;  // cannot happen
     BpLaunch l{pl->rg, pl->fp16, pl->bp_smem, pl->minb};
-    return launch_backproject(a, l, pl->d_arrived, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
+    // A call raises the counters to its number, which costs nothing (zeroing
+    // them first takes 1.5 us of a 23 us frame); a captured call runs many times
+    // with one number, so its graph zeroes them.  (Tiles of one block are never
+    // split.)
+    BpArrivals arr{pl->d_arrived, live ? ++pl->bp_calls * kArrivalStep : 0};
+    if (!live && a.blocks_per_tile > 1 &&
+        cudaMemsetAsync(pl->d_arrived, 0, (size_t)a.n_tiles * 8 * sizeof(unsigned long long), s) != cudaSuccess)
+        return SAR_ECUDA;
+    return launch_backproject(a, l, arr, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
 int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const double *q_rx, const float *fd,
@@ -1170,7 +1182,7 @@ int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const d
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return SAR_ECUDA;
     const bool live = cap == cudaStreamCaptureStatusNone;
     if (live && cudaStreamWaitEvent(s, pl->bp_done, 0) != cudaSuccess) return SAR_ECUDA;
-    const int rc = use_pairs(pl, M) ? bp_launch_pairs(pl, a, s) : bp_launch_copying(pl, a, s);
+    const int rc = use_pairs(pl, M) ? bp_launch_pairs(pl, a, s) : bp_launch_copying(pl, a, s, live);
     if (rc) return rc;
     return !live || cudaEventRecord(pl->bp_done, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
@@ -1214,7 +1226,7 @@ int backproject_with_scratch(sar_plan *pl, const void *prof, int M, const double
     BpLaunch l{pl->rg, pl->fp16, pl->bp_smem, pl->minb};
     DeviceGuard dg(pl->device);
     if (!dg.ok) return SAR_ECUDA;
-    return launch_backproject(a, l, nullptr, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
+    return launch_backproject(a, l, BpArrivals{}, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
 }  // namespace sar
@@ -2093,9 +2105,6 @@ int sar_plan_check_errors(sar_plan *pl) {
     int h[4] = {0, 0, 0, 0};
     if (cudaMemcpy(h, pl->d_err, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess) return SAR_ECUDA;
     if (cudaMemset(pl->d_err, 0, sizeof(h)) != cudaSuccess) return SAR_ECUDA;
-    if (h[0] & kErrStall)  // a launch gave up: arrivals of its split tiles are void
-        for (const sar_plan::Tiling &t : pl->tilings)
-            if (cudaMemset(t.d_arrived, 0, (size_t)t.n_tiles * 8 * sizeof(int)) != cudaSuccess) return SAR_ECUDA;
     return (h[0] & kErrStall) ? SAR_ETIMEOUT : h[0] ? SAR_EBOUNDS : SAR_OK;
 }
 

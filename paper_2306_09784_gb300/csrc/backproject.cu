@@ -594,40 +594,15 @@ __device__ __forceinline__ void process_segment(const BpArgs &a, const Smem &sm,
 }
 
 // A split tile whose share this warp has just written to `partial`: the last
-// warp to arrive for its 128 pixels adds all CTAs' shares, in CTA order.
-__device__ __forceinline__ void finish_split_tile(const BpArgs &a, int *arrived, int tile) {
-    __threadfence();
-    __syncwarp();
-    const long long PB = a.blocks_per_tile, ua = (long long)tile * PB, ub = ua + PB - 1;
-    const int ia = (int)(((ua + 1) * a.G - 1) / a.units), ib = (int)(((ub + 1) * a.G - 1) / a.units);
-    int *count = arrived + tile * (kBpThreads / 32) + (threadIdx.x >> 5);
-    int n = 0;
-    if ((threadIdx.x & 31) == 0) n = atomicAdd(count, 1);
-    n = __shfl_sync(0xffffffffu, n, 0);
-    if (n != ib - ia) return;
-    __threadfence();
-    if ((threadIdx.x & 31) == 0) *count = 0;  // for the next launch
-    float2 acc[kPxPerThread];
-#pragma unroll
-    for (int j = 0; j < kPxPerThread; ++j) acc[j] = make_float2(0.f, 0.f);
-    // CTA ia may have begun in an earlier tile; the others begin in this one
-    long long at = (long long)ia * a.seg_max + (tile - (int)((long long)ia * a.units / a.G / PB));
-#pragma unroll 4
-    for (int i = ia; i <= ib; ++i) {
-        const float2 *part = a.partial + at * kTilePx + threadIdx.x;
-        at = (long long)(i + 1) * a.seg_max;
-#pragma unroll
-        for (int j = 0; j < kPxPerThread; ++j) {
-            const float2 v = __ldcg(part + j * kBpThreads);
-            acc[j].x += v.x;
-            acc[j].y += v.y;
-        }
-    }
+// warp to arrive for its 128 pixels writes the sum of all shares.
+__device__ __forceinline__ void finish_split_tile(const BpArgs &a, const BpArrivals &arrived, int tile) {
+    float acc_re[kPxPerThread], acc_im[kPxPerThread];
+    if (!sum_split_tile(a, arrived, tile, acc_re, acc_im)) return;
 #pragma unroll
     for (int j = 0; j < kPxPerThread; ++j) {
         const int o = a.out_idx[(long long)tile * kTilePx + threadIdx.x + j * kBpThreads];
         if (o < 0) continue;
-        float2 v = acc[j];
+        float2 v = make_float2(acc_re[j], acc_im[j]);
         if (a.accumulate) {
             const float2 old = a.image[o];
             v.x += old.x;
@@ -640,11 +615,11 @@ __device__ __forceinline__ void finish_split_tile(const BpArgs &a, int *arrived,
 
 // MINB: CTAs per SM the register budget is sized for (2: 128 registers and
 // more independent updates per thread; 3: 80 registers and more warps).
-// arrived: [n_tiles][8] arrivals at split tiles, zero between launches, to sum
+// arrived: counters of the arrivals at split tiles (see sum_split_tile), to sum
 // them here (a separate fix-up launch costs a small frame 8 of its 29 us);
 // null: bp_fixup_kernel does (sar_backproject_noalloc's scratch has none).
 template <int RG, bool FP16, bool FD, int MINB>
-__global__ void __launch_bounds__(kBpThreads, MINB) backproject_kernel(BpArgs a, int *arrived) {
+__global__ void __launch_bounds__(kBpThreads, MINB) backproject_kernel(BpArgs a, BpArrivals arrived) {
     extern __shared__ __align__(16) unsigned char smem_bp[];
     Smem sm;
     sm.base = smem_bp;
@@ -665,7 +640,7 @@ __global__ void __launch_bounds__(kBpThreads, MINB) backproject_kernel(BpArgs a,
         if (!(b0 == 0 && b1 == PB))
             dst = a.partial + ((long long)blockIdx.x * a.seg_max + (tile - t_first)) * kTilePx;
         process_segment<RG, FP16, FD>(a, sm, tile, b0, b1, dst);
-        if (dst && arrived) finish_split_tile(a, arrived, tile);
+        if (dst && arrived.count) finish_split_tile(a, arrived, tile);
         u += b1 - b0;
     }
 }
@@ -1008,14 +983,14 @@ cudaError_t launch_batch_fixup(const BpMultiArgs &m, const BpCheck &chk, int tot
     return cudaGetLastError();
 }
 
-cudaError_t launch_backproject(const BpArgs &a, const BpLaunch &l, int *arrived, cudaStream_t s) {
+cudaError_t launch_backproject(const BpArgs &a, const BpLaunch &l, BpArrivals arrived, cudaStream_t s) {
     void *k = select_kernel(l.rg, l.fp16, a.fdopp != nullptr, l.minb);
     if (!k) return cudaErrorInvalidValue;
     if (a.units == 0) return cudaSuccess;
     BpArgs args = a;
     void *params[] = {&args, &arrived};
     cudaError_t e = cudaLaunchKernel(k, dim3(a.G), dim3(kBpThreads), params, l.smem, s);
-    if (e != cudaSuccess || arrived) return e;
+    if (e != cudaSuccess || arrived.count) return e;
     bp_fixup_kernel<<<a.n_tiles, kFixupThreads, 0, s>>>(a);
     return cudaGetLastError();
 }

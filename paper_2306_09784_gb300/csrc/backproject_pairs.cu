@@ -575,36 +575,11 @@ __device__ __forceinline__ bool pair_segment(const BpPairArgs &pa, PairSmem &sm,
 
     if (!whole) {
         // this CTA's share of a split tile; the last warp to arrive for these
-        // 128 pixels adds all shares in CTA order
+        // 128 pixels adds all shares
         float2 *dst = a.partial + (long long)slot * kTilePx + threadIdx.x;
 #pragma unroll
         for (int j = 0; j < kPxPerThread; ++j) __stcg(dst + j * kBpThreads, make_float2(acc_re[j], acc_im[j]));
-        __threadfence();
-        __syncwarp();
-        const long long PB = a.blocks_per_tile, ua = (long long)tile * PB, ub = ua + PB - 1;
-        const int ia = (int)(((ua + 1) * a.G - 1) / a.units), ib = (int)(((ub + 1) * a.G - 1) / a.units);
-        int *arrived = pa.arrived + tile * kWarps + (threadIdx.x >> 5);
-        int n = 0;
-        if ((threadIdx.x & 31) == 0) n = atomicAdd(arrived, 1);
-        n = __shfl_sync(0xffffffffu, n, 0);
-        if (n != ib - ia) return true;
-        __threadfence();
-        if ((threadIdx.x & 31) == 0) *arrived = 0;  // for the next launch
-#pragma unroll
-        for (int j = 0; j < kPxPerThread; ++j) acc_re[j] = acc_im[j] = 0.f;
-        // CTA ia may have begun in an earlier tile; the others begin in this one
-        long long at = (long long)ia * a.seg_max + (tile - (int)((long long)ia * a.units / a.G / PB));
-#pragma unroll 4
-        for (int i = ia; i <= ib; ++i) {
-            const float2 *part = a.partial + at * kTilePx + threadIdx.x;
-            at = (long long)(i + 1) * a.seg_max;
-#pragma unroll
-            for (int j = 0; j < kPxPerThread; ++j) {
-                const float2 v = __ldcg(part + j * kBpThreads);
-                acc_re[j] += v.x;
-                acc_im[j] += v.y;
-            }
-        }
+        if (!sum_split_tile(a, pa.arrived, tile, acc_re, acc_im)) return true;
     }
 #pragma unroll
     for (int j = 0; j < kPxPerThread; ++j) {
@@ -661,9 +636,11 @@ __global__ void __launch_bounds__(kBpThreads, MINB)
 // row, 16 bytes written per bin.  The warp of a pulse's first row also takes
 // the pulse's Rx offsets o = q_rx - q_tx (FP64 differences, FP32 values), their
 // largest square, and into call[0], call[1] (zero before the launch) the FP32
-// bits of the call's largest |o| and whether any o has a y component.
+// bits of the call's largest |o| and whether any o has a y component.  The
+// launch also zeroes the arrival counters of the call's split tiles.
 template <bool FP16>
 __global__ void __launch_bounds__(256) expand_pairs_kernel(ExpandArgs e) {
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < e.n_arrived; i += gridDim.x * 256) e.arrived[i] = 0;
     __shared__ unsigned call_sh[2];
     if (threadIdx.x < 2) call_sh[threadIdx.x] = 0;
     __syncthreads();

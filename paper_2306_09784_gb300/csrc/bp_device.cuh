@@ -149,5 +149,44 @@ __device__ __forceinline__ void accumulate2(float2 idx, uint32_t ac, float2 kap,
     acc_imb[2 * h + 1] = imb.y;
 }
 
+// Arrival of a warp that has just written its CTA's share of a split tile (its
+// 128 pixels) to `partial`.  The last of the tile's CTAs to arrive gets the sum
+// of all shares, in CTA order, and true.  arr.count: [n_tiles][8] counters that
+// this launch finds at zero (arr.base = 0), or that it raises to its own base,
+// above every count of an earlier call: nothing an earlier call left behind
+// (one that gave up, or calls that overlapped) reaches this one.
+__device__ __forceinline__ bool sum_split_tile(const BpArgs &a, const BpArrivals &arr, int tile,
+                                               float (&acc_re)[kPxPerThread], float (&acc_im)[kPxPerThread]) {
+    __threadfence();
+    __syncwarp();
+    const long long PB = a.blocks_per_tile, ua = (long long)tile * PB, ub = ua + PB - 1;
+    const int ia = (int)(((ua + 1) * a.G - 1) / a.units), ib = (int)(((ub + 1) * a.G - 1) / a.units);
+    int n = 0;
+    if ((threadIdx.x & 31) == 0) {
+        unsigned long long *count = arr.count + tile * (kBpThreads / 32) + (threadIdx.x >> 5);
+        if (arr.base) atomicMax(count, arr.base);
+        n = (int)(atomicAdd(count, 1ull) - arr.base);
+    }
+    n = __shfl_sync(0xffffffffu, n, 0);
+    if (n != ib - ia) return false;
+    __threadfence();
+#pragma unroll
+    for (int j = 0; j < kPxPerThread; ++j) acc_re[j] = acc_im[j] = 0.f;
+    // CTA ia may have begun in an earlier tile; the others begin in this one
+    long long at = (long long)ia * a.seg_max + (tile - (int)((long long)ia * a.units / a.G / PB));
+#pragma unroll 4
+    for (int i = ia; i <= ib; ++i) {
+        const float2 *part = a.partial + at * kTilePx + threadIdx.x;
+        at = (long long)(i + 1) * a.seg_max;
+#pragma unroll
+        for (int j = 0; j < kPxPerThread; ++j) {
+            const float2 v = __ldcg(part + j * kBpThreads);
+            acc_re[j] += v.x;
+            acc_im[j] += v.y;
+        }
+    }
+    return true;
+}
+
 }  // namespace
 }  // namespace sar

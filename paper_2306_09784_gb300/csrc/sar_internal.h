@@ -177,6 +177,14 @@ struct BpLaunch {
     int minb;     // CTAs per SM the kernel's registers are sized for (2 or 3)
 };
 
+// Counters of the arrivals at split tiles, 8 per tile (one per warp's pixels).
+// They start at zero with base = 0, or anywhere below base, a multiple of
+// kArrivalStep that no earlier launch on them reached.
+constexpr unsigned long long kArrivalStep = 1ull << 16;  // above the CTAs of a launch
+struct BpArrivals {
+    unsigned long long *count = nullptr, base = 0;
+};
+
 // Backprojection from interpolation pairs (backproject_pairs.cu).
 constexpr int kPairUnit = 2;  // pulses per work unit
 constexpr int kWaitPolls = 1 << 20;  // polls of a wait for a copy: far longer than any takes
@@ -189,7 +197,7 @@ struct BpPairArgs {
     const float4 *rx;          // [M R] Rx offset (o_x, o_y, |o|^2, 0)
     const float *o2max;        // [M] largest |o|^2 of the pulse
     const unsigned *call;      // FP32 bits of the call's largest |o|; any o_y
-    int *arrived;              // [n_tiles][8] warps done with a split tile's pixels, zero between launches
+    BpArrivals arrived;        // warps done with a split tile's pixels
     unsigned smem_bytes;       // dynamic shared memory of the launch
     int mb_cap;                // chirps per pipeline block at most
     int polls;                 // polls of a copy's barrier before the call gives up
@@ -202,6 +210,8 @@ struct ExpandArgs {
     float4 *rx;
     float *o2max;
     unsigned *call;
+    unsigned long long *arrived;  // zeroed by the launch
+    int n_arrived;
     int rows, R, n_bins;
     float2 cb_k;
     float inv_kappa;
@@ -213,9 +223,9 @@ cudaError_t launch_backproject_pairs(const BpPairArgs &pa, const ExpandArgs &e, 
 size_t bp_smem_bytes(int Mb, int R, int L, bool fp16);
 cudaError_t bp_prepare(bool fp16, int rg, size_t smem);  // sets function attributes
 int bp_occupancy(bool fp16, int rg, size_t smem, int minb, int *ctas_per_sm);
-// arrived: zeroed counters (8 per tile) to sum split tiles in the same launch;
-// null: by a fix-up launch.
-cudaError_t launch_backproject(const BpArgs &a, const BpLaunch &l, int *arrived, cudaStream_t s);
+// arrived: counters to sum split tiles in the same launch; null: by a fix-up
+// launch.
+cudaError_t launch_backproject(const BpArgs &a, const BpLaunch &l, BpArrivals arrived, cudaStream_t s);
 cudaError_t bp_batch_prepare(int rg, bool fp16, size_t smem, int *ctas_per_sm);
 // host_jobs: the class's jobs in host memory (the same as c.jobs), passed as
 // parameters when there are at most kParamJobs; null to read c.jobs.

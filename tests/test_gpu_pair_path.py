@@ -93,3 +93,36 @@ def test_wait_that_runs_out_is_reported():
     got = plan.backproject(prof, M, qt, qr)
     assert plan.check_errors() == sar.SAR_OK
     assert torch.equal(got, ref)
+
+
+def test_nothing_is_left_behind_by_a_call_that_gave_up():
+    """Split tiles are counted per call: after calls that gave up (no status
+    read in between), after a captured call and across both kernels and chirp
+    counts, each call equals its own first result bit for bit."""
+    import torch
+    M, small = 600, 90
+    plan, prof, qt, qr, _ = _frames(4, M, synth.Grid(-4.1, 1.2, 0.033, 0.03, 250, 270))
+    assert plan.pair_path(M)[0] and not plan.pair_path(small)[0]
+    beat = torch.randn(small, 4, 256, dtype=torch.complex64, device="cuda",
+                       generator=torch.Generator("cuda").manual_seed(2))
+    prof_s, qt_s, qr_s = plan.range_compress(beat), qt[:small].contiguous(), qr[:small].contiguous()
+    calls = {M: (prof, M, qt, qr), small: (prof_s, small, qt_s, qr_s), 41: (prof_s, 41, qt_s, qr_s)}
+    ref = {n: plan.backproject(*c).clone() for n, c in calls.items()}
+    img = torch.zeros_like(ref[M])
+    torch.cuda.synchronize()
+    graphs, stream = {}, torch.cuda.Stream()
+    for n, c in calls.items():
+        graphs[n] = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graphs[n], stream=stream):
+            plan.backproject(*c, image=img, stream=stream)
+    for n in (small, M, 41, M, small, 41):
+        plan.set_wait_limit(0)
+        plan.backproject(*calls[M])
+        plan.set_wait_limit()
+        got = plan.backproject(*calls[n])
+        assert torch.equal(got, ref[n]), n
+        img.zero_()
+        graphs[n].replay()
+        assert torch.equal(img, ref[n]), n
+        for k in (41, small, M):  # and ordinary calls after the replay
+            assert torch.equal(plan.backproject(*calls[k]), ref[k]), (n, k)

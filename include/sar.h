@@ -262,8 +262,13 @@ int sar_range_spectrum(sar_plan *plan, const void *beat_dev, int32_t M,
  * device_bytes; sar_plan_pair_path tells which calls).  A plan goes without it
  * where no call of its sizes would gain, where it would take over 1 GiB or a
  * sixteenth of the free memory, or where its HBM budget would not hold the
- * buffers allocated later.  A call on another stream than the previous one
- * waits for it.
+ * buffers allocated later.
+ * Backprojections of one plan share its scratch.  A call waits for the plan's
+ * previous one, whichever stream that ran on.  A captured call takes no part
+ * in this: the caller orders its replays against each other and against every
+ * other backprojection of the plan, and branches of one graph likewise (one
+ * stream or events).  Calls that overlap all the same spoil each other's
+ * images and may be flagged SAR_EBOUNDS; later calls are not affected.
  */
 int sar_backproject(sar_plan *plan, const void *prof_dev, int32_t M,
                     const double *q_tx_dev, const double *q_rx_dev,

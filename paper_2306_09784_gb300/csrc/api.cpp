@@ -27,6 +27,9 @@ constexpr int kMaxPulsesPerBlock = 32;
 constexpr size_t kPairSmem[2] = {113 * 1024, 75 * 1024};
 // Largest workspace of interpolation pairs a plan keeps.
 constexpr size_t kPairBytesMax = size_t(1) << 30;
+// Call words of a plan: one slot for the calls enqueued directly, which are
+// ordered, and one for each captured call (shared from the 1024th on).
+constexpr unsigned kCallSlots = 1024;
 // GPU time (ps) that the pair kernel saves per window (pixel tile x chirp x Rx)
 // of L bins, and spends, against the copying kernel (see pairs_pay).
 constexpr double kPairPerWindow = 52.0, kPairPerWindowBin = 3.8, kPairPerPulseTile = 365.0;
@@ -59,7 +62,8 @@ struct sar_plan {
     float4 *d_pairs = nullptr, *d_rx = nullptr, *d_zero = nullptr;
     float *d_o2max = nullptr;
     int zero_len = 0;
-    unsigned *d_call = nullptr;
+    unsigned *d_call = nullptr;  // [kCallSlots][4]
+    unsigned captures = 0;       // captured calls so far
     // the end of the last backprojection: calls share the plan's pairs,
     // partial sums and arrival counters, so that one on another stream waits
     cudaEvent_t bp_done = nullptr;
@@ -728,10 +732,11 @@ void add_pair_workspace(sar_plan *pl) {
         const size_t retile = pl->tile_w ? 2 * tiles * (kTilePx * 20 + sizeof(TileInfo)) +
                                                12 * (size_t)pl->num_sms * kTilePx * 8 + 8 * 256
                                          : 0;
-        if (pl->used + bytes + geo + (size_t)zero_len * 16 + 1024 + host + retile > pl->budget) return;
+        if (pl->used + bytes + geo + (size_t)zero_len * 16 + kCallSlots * 16 + 1024 + host + retile > pl->budget) return;
     }
     // one block: call words, zeros, Rx offsets and their largest squares
-    const size_t rx_o = 256 + (size_t)zero_len * sizeof(float4);
+    const size_t zero_o = kCallSlots * 4 * sizeof(unsigned);
+    const size_t rx_o = zero_o + (size_t)zero_len * sizeof(float4);
     void *small = nullptr, *pairs = nullptr;
     if (dev_alloc(pl, rx_o + geo, &small) || dev_alloc(pl, bytes, &pairs) ||
         cudaMemset(small, 0, rx_o) != cudaSuccess ||
@@ -742,7 +747,7 @@ void add_pair_workspace(sar_plan *pl) {
     pl->d_pairs = (float4 *)pairs;
     pl->pair_bytes = bytes + rx_o + geo;
     pl->d_call = (unsigned *)small;
-    pl->d_zero = (float4 *)((char *)small + 256);
+    pl->d_zero = (float4 *)((char *)small + zero_o);
     pl->zero_len = zero_len;
     pl->d_rx = (float4 *)((char *)small + rx_o);
     pl->d_o2max = (float *)(pl->d_rx + rows);
@@ -1089,8 +1094,9 @@ bool use_pairs(const sar_plan *pl, int M) {
     return pl->d_pairs && pl->L <= pl->zero_len && pairs_pay(pl, M);
 }
 
-// Backprojection from interpolation pairs of a call's arguments a.
-int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
+// Backprojection from interpolation pairs of a call's arguments a.  live:
+// enqueued now, not captured.
+int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s, bool live) {
     BpPairArgs pa{};
     a.blocks_per_tile = (a.M + kPairUnit - 1) / kPairUnit;
     a.units = (long long)a.n_tiles * a.blocks_per_tile;
@@ -1104,7 +1110,10 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
     pa.zero = pl->d_zero;
     pa.rx = pl->d_rx;
     pa.o2max = pl->d_o2max;
-    pa.call = pl->d_call;
+    // The kernel's layout follows from the call's words, so no other call may
+    // write them while it runs: a captured call has its own
+    unsigned *call = pl->d_call + (live ? 0u : 4u * (1 + pl->captures++ % (kCallSlots - 1)));
+    pa.call = call;
     pa.arrived = BpArrivals{pl->d_arrived, 0};
     pa.div_blk = ((1ull << 32) + (unsigned)a.Mb - 1) / (unsigned)a.Mb;
     pa.smem_bytes = (unsigned)pl->pair_smem;
@@ -1118,7 +1127,7 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
     e.pairs = pl->d_pairs;
     e.rx = pl->d_rx;
     e.o2max = pl->d_o2max;
-    e.call = pl->d_call;
+    e.call = call;
     e.arrived = pl->d_arrived;
     e.n_arrived = a.n_tiles * 8;
     e.rows = a.M * a.R;
@@ -1129,12 +1138,11 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s) {
     const BpLaunch l{pl->rg, pl->fp16, pl->pair_smem, pl->minb};
     // the call's words start from zero here, not by the call's number: a
     // captured call runs many times
-    if (cudaMemsetAsync(pl->d_call, 0, 16, s) != cudaSuccess) return SAR_ECUDA;
+    if (cudaMemsetAsync(call, 0, 16, s) != cudaSuccess) return SAR_ECUDA;
     return launch_backproject_pairs(pa, e, l, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
-// Backprojection of a call's arguments a by the copying kernel.  live: enqueued
-// now, not captured.
+// Backprojection of a call's arguments a by the copying kernel.
 int bp_launch_copying(sar_plan *pl, BpArgs a, cudaStream_t s, bool live) {
     // a call too small for the pair kernel cuts its pulse blocks so that the
     // CTAs' counts of them even out: the block that minimises, in windows'
@@ -1182,7 +1190,7 @@ int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const d
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return SAR_ECUDA;
     const bool live = cap == cudaStreamCaptureStatusNone;
     if (live && cudaStreamWaitEvent(s, pl->bp_done, 0) != cudaSuccess) return SAR_ECUDA;
-    const int rc = use_pairs(pl, M) ? bp_launch_pairs(pl, a, s) : bp_launch_copying(pl, a, s, live);
+    const int rc = use_pairs(pl, M) ? bp_launch_pairs(pl, a, s, live) : bp_launch_copying(pl, a, s, live);
     if (rc) return rc;
     return !live || cudaEventRecord(pl->bp_done, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }

@@ -84,11 +84,11 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_
 // three slots of Tx records and two of Rx records.
 struct PairLayout {
     int Mt, slots, Lt, s0;
-    uint32_t table, txr, rxa, txc, rxb;
+    uint32_t table, txr, rxa, txc, rxb, txo;
 };
 
 // Bytes of the records of one pulse.
-__host__ __device__ constexpr unsigned pair_const_bytes(int R) { return 3u * 24u + 2u * 24u * (unsigned)R; }
+__host__ __device__ constexpr unsigned pair_const_bytes(int R) { return 3u * 28u + 2u * 24u * (unsigned)R; }
 
 // PU: pulses the pixel loop unrolls together (blocks are multiples of it
 // where they can be).
@@ -125,6 +125,7 @@ __device__ __forceinline__ PairLayout pair_layout(const BpPairArgs &pa, const Ti
     l.rxa = l.txr + 3u * l.Mt * 16u;
     l.txc = l.rxa + 2u * l.Mt * a.R * 16u;
     l.rxb = l.txc + 3u * l.Mt * 8u;
+    l.txo = l.rxb + 2u * l.Mt * a.R * 8u;
     return l;
 }
 
@@ -136,6 +137,8 @@ struct PairSmem {
     // constant bits, k_lo)
     __device__ float4 *txr(int s) const { return reinterpret_cast<float4 *>(base + l.txr) + s * l.Mt; }
     __device__ int2 *txc(int s) const { return reinterpret_cast<int2 *>(base + l.txc) + s * l.Mt; }
+    // largest |o|^2 that the pulse's window and loop choice cover
+    __device__ float *txo(int s) const { return reinterpret_cast<float *>(base + l.txo) + s * l.Mt; }
     // Rx records of slot t (b % 2).  Expansion loop: (o_x / 2, -c / 2) and
     // o_y / 2; exact loop: (wx, wy, R, R^2) and (index constant bits, k_lo)
     __device__ float4 *rxa(int t, int R) const { return reinterpret_cast<float4 *>(base + l.rxa) + t * l.Mt * R; }
@@ -194,10 +197,11 @@ __device__ __forceinline__ void prep_tx(const BpPairArgs &pa, const PairSmem &sm
                 t4 = make_float4((float)wx, (float)wy, r_f, (float)r2);
                 const int k_lo = __double2int_rd(fma(2.0 * a.a1, r_tx, -(double)ti.klo_off)) - kGuardBins;
                 c = make_int2(__float_as_int((float)fma(2.0 * a.a1, r_tx, -(double)k_lo)), k_lo);
-                exact = pulse_exact(ti, tol2, t4.x, t4.y, o2);
+                exact = pulse_exact(ti, tol2, t4.x, t4.y, o2) || !(sqrtf(o2) <= __uint_as_float(pa.call[0]));
             }
             sm.txr(s)[lane] = t4;
             sm.txc(s)[lane] = c;
+            sm.txo(s)[lane] = o2;
             if (exact) bits = 1u << (fast_div(m, pa.div_blk) - run0);
         }
     } else {
@@ -223,6 +227,10 @@ __device__ __forceinline__ int run_of(const BpPairArgs &pa, int m0, int p) {
 // Rx records of pulses [m0, m0 + np) (Tx slot s) into slot t: the expansion
 // loop's FP32 coefficients, or for pulses on the exact loop the FP64 Rx
 // reference range, window start and index (prep_exact in backproject.cu).
+// The offsets of the expansion loop come from memory that every call of the plan
+// writes.  Calls are ordered, but a replayed graph's are ordered by the caller;
+// so that a mistake there spoils an image and no more, an offset that the
+// pulse's window and loop choice do not cover is dropped and flagged.
 template <bool MULTI, int RG>
 __device__ __forceinline__ void prep_rx(const BpPairArgs &pa, const PairSmem &sm, const TileInfo &ti, int m0, int np,
                                         int s, int t, unsigned exact) {
@@ -231,12 +239,18 @@ __device__ __forceinline__ void prep_rx(const BpPairArgs &pa, const PairSmem &sm
     const float4 *txr = sm.txr(s);
     float4 *rxa = sm.rxa(t, R);
     int2 *rxb = sm.rxb(t, R);
+    const float *txo = sm.txo(s);
+    const bool axis = !pa.call[1];
     for (int task = threadIdx.x; task < np * R; task += kBpThreads) {
         const int p = MULTI ? fast_div(task, a.div_r) : task / RG;
         const long long row = (long long)m0 * R + task;
         if (!exact || !((exact >> run_of(pa, m0, p)) & 1u)) {
             const float4 t4 = txr[p];
-            const float4 g = pa.rx[row];  // (o_x, o_y, |o|^2, 0)
+            float4 g = pa.rx[row];  // (o_x, o_y, |o|^2, |o|^2 or infinite off the x axis)
+            if (!((axis ? g.w : g.z) <= txo[p])) {
+                g = make_float4(0.f, 0.f, 0.f, 0.f);
+                atomicOr(a.err, kErrGeometry);
+            }
             const float cexp = fmaf(0.5f, g.z, -fmaf(t4.x, g.x, t4.y * g.y));
             // halved so that the pixel loop gets -a / 2 directly
             rxa[task] = make_float4(0.5f * g.x, -0.5f * cexp, 0.f, 0.f);
@@ -656,7 +670,7 @@ __global__ void __launch_bounds__(256) expand_pairs_kernel(ExpandArgs e) {
                 const double2 qr = reinterpret_cast<const double2 *>(e.q_rx)[row + r];
                 const float ox = (float)(qr.x - qt.x), oy = (float)(qr.y - qt.y);
                 const float o2 = fmaf(ox, ox, oy * oy);
-                e.rx[row + r] = make_float4(ox, oy, o2, 0.f);
+                e.rx[row + r] = make_float4(ox, oy, o2, fabsf(oy) <= 1e-9f ? o2 : INFINITY);
                 o2max = fmaxf(o2max, o2 < INFINITY ? o2 : INFINITY);  // NaN: out of the expansion loop's reach
                 off |= !(fabsf(oy) <= 1e-9f);
             }

@@ -194,9 +194,9 @@ struct BpPairArgs {
     unsigned long long div_blk;  // ceil(2^32 / Mb)
     const float4 *pairs;       // [M R][n_bins] (A, D) of bins crop_lo ... (the last one of a row unused)
     const float4 *zero;        // L zero entries
-    const float4 *rx;          // [M R] Rx offset (o_x, o_y, |o|^2, 0)
+    const float4 *rx;          // [M R] Rx offset (o_x, o_y, |o|^2, the same or infinite if o_y != 0)
     const float *o2max;        // [M] largest |o|^2 of the pulse
-    const unsigned *call;      // FP32 bits of the call's largest |o|; any o_y
+    const unsigned *call;      // FP32 bits of the call's largest |o|; any o_y (no other call writes these)
     BpArrivals arrived;        // warps done with a split tile's pixels
     unsigned smem_bytes;       // dynamic shared memory of the launch
     int mb_cap;                // chirps per pipeline block at most

@@ -126,3 +126,47 @@ def test_nothing_is_left_behind_by_a_call_that_gave_up():
         assert torch.equal(img, ref[n]), n
         for k in (41, small, M):  # and ordinary calls after the replay
             assert torch.equal(plan.backproject(*calls[k]), ref[k]), (n, k)
+
+
+@pytest.mark.parametrize("M0,M1", [(1101, 620), (90, 47)])  # on the pair path, and below its line
+def test_calls_on_several_streams_and_ordered_replays(M0, M1):
+    """Calls of one plan with different chirps, profiles and arrays alternate on
+    two streams, then with replays of captured calls that the caller orders by
+    events: every image is its call's own, bit for bit."""
+    import torch
+    plan, prof, qt, qr, _ = _frames(4, M0, synth.Grid(-4.1, 1.2, 0.033, 0.03, 250, 270))
+    beat = torch.randn(M1, 4, 256, dtype=torch.complex64, device="cuda",
+                       generator=torch.Generator("cuda").manual_seed(3))
+    qt1 = qt[:M1].flip(0).contiguous()
+    qr1 = (qt1[:, None, :] + 2.5 * (qr[:M1] - qt[:M1, None, :])).contiguous()
+    frames = [(prof, M0, qt, qr), (plan.range_compress(beat), M1, qt1, qr1)]
+    assert [plan.pair_path(f[1])[0] for f in frames] == [M0 > 500] * 2
+    ref = [plan.backproject(*f).clone() for f in frames]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    outs = [torch.zeros_like(ref[0]) for _ in range(8)]
+    for i, o in enumerate(outs):
+        plan.backproject(*frames[i % 2], image=o, stream=streams[(i + i // 4) % 2])
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, ref[i % 2]) for i, o in enumerate(outs))
+    img, graph = torch.zeros_like(ref[0]), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=streams[0]):
+        plan.backproject(*frames[0], image=img, stream=streams[0])
+    for i, o in enumerate(outs):
+        img.zero_(), o.zero_()
+        torch.cuda.synchronize()
+        ev = torch.cuda.Event()
+        if i % 2:  # the replay, then the call
+            with torch.cuda.stream(streams[0]):
+                graph.replay()
+            ev.record(streams[0])
+            ev.wait(streams[1])
+            plan.backproject(*frames[1], image=o, stream=streams[1])
+        else:  # the call, then the replay
+            plan.backproject(*frames[1], image=o, stream=streams[1])
+            ev.record(streams[1])
+            ev.wait(streams[0])
+            with torch.cuda.stream(streams[0]):
+                graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(img, ref[0]) and torch.equal(o, ref[1])

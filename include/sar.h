@@ -291,8 +291,11 @@ int sar_backproject(sar_plan *plan, const void *prof_dev, int32_t M,
  *  fdopp_idx_dev  float [n_pixels] output in image order, ready for
  *             sar_backproject; |f_doppler| <= 2 f0' |vbar| N_fft / (c fs), so a
  *             plan with max_doppler_bins at least that takes every pixel
- * Asynchronous on `stream` (two kernels, device memory only).  SAR_EINVAL for
- * null or misaligned pointers or M outside 1..max_pulses.
+ * Asynchronous on `stream` (two kernels, device memory only).  Calls of one
+ * plan share its scratch and are ordered as backprojections are: a call waits
+ * for the previous one on any stream, replays of captured calls are ordered by
+ * the caller.  SAR_EINVAL for null or misaligned pointers or M outside
+ * 1..max_pulses.
  */
 int sar_doppler_offsets(sar_plan *plan, const double *q_tx_dev, const double *q_rx_dev,
                         const double *vel_dev, int32_t M, float *fdopp_idx_dev, void *stream);

@@ -64,9 +64,10 @@ struct sar_plan {
     int zero_len = 0;
     unsigned *d_call = nullptr;  // [kCallSlots][4]
     unsigned captures = 0;       // captured calls so far
-    // the end of the last backprojection: calls share the plan's pairs,
-    // partial sums and arrival counters, so that one on another stream waits
-    cudaEvent_t bp_done = nullptr;
+    // the end of the last backprojection (calls share the plan's pairs, partial
+    // sums and arrival counters) and of the last Doppler offsets (partial sums):
+    // a call on another stream waits (see CallOrder)
+    cudaEvent_t bp_done = nullptr, doppler_done = nullptr;
     size_t pair_smem = 0, pair_bytes = 0;
     int polls = kWaitPolls;  // of the pair kernel's waits for its copies
     int pair_G = 0, mb_cap = kMaxPulsesPerBlock;
@@ -248,7 +249,7 @@ void free_plan(sar_plan *pl) {
     cudaDeviceSynchronize();
     for (void *p : pl->allocs) cudaFree(p);
     if (pl->s_copy) cudaStreamDestroy(pl->s_copy);
-    for (cudaEvent_t e : {pl->ev_start, pl->ev_chunk[0], pl->ev_chunk[1], pl->ev_traj, pl->bp_done})
+    for (cudaEvent_t e : {pl->ev_start, pl->ev_chunk[0], pl->ev_chunk[1], pl->ev_traj, pl->bp_done, pl->doppler_done})
         if (e) cudaEventDestroy(e);
     delete pl;
 }
@@ -936,11 +937,12 @@ int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t bud
         free_plan(pl);
         return rc;
     }
-    if (cudaEventCreateWithFlags(&pl->bp_done, cudaEventDisableTiming) != cudaSuccess) {
-        pl->bp_done = nullptr;
-        free_plan(pl);
-        return SAR_ECUDA;
-    }
+    for (cudaEvent_t *e : {&pl->bp_done, &pl->doppler_done})
+        if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) {
+            *e = nullptr;
+            free_plan(pl);
+            return SAR_ECUDA;
+        }
     add_pair_workspace(pl);
     recall_shape(pl);
     *out = pl;
@@ -1176,6 +1178,25 @@ int bp_launch_copying(sar_plan *pl, BpArgs a, cudaStream_t s, bool live) {
     return launch_backproject(a, l, arr, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
 }
 
+// Orders a call after the last one that shared its scratch, whichever stream
+// that ran on: handles do not tell streams apart (reuse, per-thread default
+// streams), and on the same stream the wait is free.  A captured call takes no
+// part: its graph's launches are ordered by the caller.
+struct CallOrder {
+    cudaEvent_t done = nullptr;
+    cudaStream_t s = nullptr;
+    bool live = true;
+    bool begin(cudaEvent_t last, cudaStream_t stream) {
+        done = last;
+        s = stream;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return false;
+        live = cap == cudaStreamCaptureStatusNone;
+        return !live || cudaStreamWaitEvent(s, done, 0) == cudaSuccess;
+    }
+    bool end() const { return !live || cudaEventRecord(done, s) == cudaSuccess; }
+};
+
 int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const double *q_rx, const float *fd,
               void *image, int accumulate, cudaStream_t s, int m0 = 0, int M_tot = 0,
               void *image_out = nullptr) {
@@ -1183,16 +1204,11 @@ int bp_launch(sar_plan *pl, const void *prof, int M, const double *q_tx, const d
     a.image_out = (float2 *)image_out;
     DeviceGuard dg(pl->device);
     if (!dg.ok) return SAR_ECUDA;
-    // order after the last call, whichever stream that ran on: handles do not
-    // tell streams apart (reuse, per-thread default streams), and on the same
-    // stream the wait is free (a captured call is ordered by its graph)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return SAR_ECUDA;
-    const bool live = cap == cudaStreamCaptureStatusNone;
-    if (live && cudaStreamWaitEvent(s, pl->bp_done, 0) != cudaSuccess) return SAR_ECUDA;
-    const int rc = use_pairs(pl, M) ? bp_launch_pairs(pl, a, s, live) : bp_launch_copying(pl, a, s, live);
+    CallOrder order;
+    if (!order.begin(pl->bp_done, s)) return SAR_ECUDA;
+    const int rc = use_pairs(pl, M) ? bp_launch_pairs(pl, a, s, order.live) : bp_launch_copying(pl, a, s, order.live);
     if (rc) return rc;
-    return !live || cudaEventRecord(pl->bp_done, s) == cudaSuccess ? SAR_OK : SAR_ECUDA;
+    return order.end() ? SAR_OK : SAR_ECUDA;
 }
 
 }  // namespace
@@ -1352,7 +1368,10 @@ int sar_doppler_offsets(sar_plan *pl, const double *q_tx_dev, const double *q_rx
     a.fd = fdopp_idx_dev;
     DeviceGuard dg(pl->device);
     if (!dg.ok) return SAR_ECUDA;
-    return launch_doppler_offsets(a, (cudaStream_t)stream) == cudaSuccess ? SAR_OK : SAR_ECUDA;
+    CallOrder order;
+    if (!order.begin(pl->doppler_done, (cudaStream_t)stream)) return SAR_ECUDA;
+    if (launch_doppler_offsets(a, (cudaStream_t)stream) != cudaSuccess) return SAR_ECUDA;
+    return order.end() ? SAR_OK : SAR_ECUDA;
 }
 
 int sar_form_image_host(sar_plan *pl, const void *beat_host, int32_t M, const float *w_az_host,

@@ -173,9 +173,11 @@ typedef struct sar_plan_info {
     int64_t n_pixels;           /* image size in complex64 values */
     int32_t n_tiles;            /* pixel tiles of 1024 reconstruction points (slots) */
     int32_t window_bins;        /* bins staged per (tile, chirp, Rx) */
-    int32_t pulses_per_block;   /* chirps staged per pipeline step (calls that take the pair path, see
-                                   sar_backproject, stage as many as fit when this is the largest block) */
-    int32_t bp_ctas;            /* persistent backprojection grid size */
+    int32_t pulses_per_block;   /* chirps staged per pipeline step.  A new plan has the largest block that
+                                   fits two CTAs per SM, and each call then chooses: on the pair path (see
+                                   sar_backproject) as many chirps as fit, in small calls fewer, so that all
+                                   CTAs do the same */
+    int32_t bp_ctas;            /* persistent grid size of calls that do not take the pair path */
     double bins_per_metre;      /* a1 = mu N_fft / (c fs) */
     double cycles_per_bin;      /* f0 / (c a1) */
     size_t device_bytes;        /* device memory the plan owns */
@@ -564,7 +566,11 @@ int sar_plan_autotune(sar_plan *plan, const void *prof_dev, int32_t M, const dou
  * sar_plan_get_info after sar_plan_autotune:
  *  rx_group          Rx channels per inner-loop group: 1..4, dividing n_rx
  *  regs_ctas_per_sm  2 or 3 (register budget of the kernel variant)
- *  pulses_per_block  chirps staged per pipeline step, 1..32
+ *  pulses_per_block  chirps staged per pipeline step, 1..32.  Every call keeps
+ *                    it, with one exception: the largest block that fits
+ *                    regs_ctas_per_sm CTAs per SM (what a new plan has and what
+ *                    sar_plan_autotune may report) leaves the choice to each
+ *                    call, as sar_plan_info describes
  * SAR_EINVAL if the shape is out of range or its shared memory does not
  * allow one CTA per SM; the plan keeps its previous shape then.  Results do
  * not depend on the shape beyond FP32 summation order.  Not thread-safe

@@ -58,7 +58,7 @@ struct sar_plan {
     float fd_max = 0.f;
     // backprojection from interpolation pairs (backproject_pairs.cu): the
     // workspace, when the plan has one, and the launch that goes with rg and
-    // minb.  mb_cap: chirps per pipeline block at most (explicit blocks only)
+    // minb
     float4 *d_pairs = nullptr, *d_rx = nullptr, *d_zero = nullptr;
     float *d_o2max = nullptr;
     int zero_len = 0;
@@ -70,7 +70,10 @@ struct sar_plan {
     cudaEvent_t bp_done = nullptr, doppler_done = nullptr;
     size_t pair_smem = 0, pair_bytes = 0;
     int polls = kWaitPolls;  // of the pair kernel's waits for its copies
-    int pair_G = 0, mb_cap = kMaxPulsesPerBlock;
+    int pair_G = 0;
+    // Mb is the block a plan starts with (or the largest that fits minb CTAs per
+    // SM): each call chooses its own; any other block is kept as it is
+    bool block_free = true;
     // device memory owned by the plan
     float *d_wr = nullptr;
     float2 *d_tw = nullptr;
@@ -265,6 +268,16 @@ int largest_block(const sar_plan *pl, int L, int minb) {
     return Mb;
 }
 
+// The pulse block a plan or tiling starts with: the largest whose shared memory
+// fits two CTAs per SM (or one less).
+int default_block(const sar_plan *pl, int L) {
+    const int R = pl->p.n_rx;
+    const size_t per_pulse = bp_smem_bytes(1, R, L, pl->fp16);
+    int Mb = (int)std::min<size_t>(kMaxPulsesPerBlock, std::max<size_t>(1, kBpSmemTarget / per_pulse));
+    while (Mb > 1 && bp_smem_bytes(Mb, R, L, pl->fp16) > kBpSmemTarget) --Mb;
+    return Mb;
+}
+
 // The pair kernel's launch for this Rx group and register budget (the current
 // tiling); false where it does not fit.
 bool pair_launch(const sar_plan *pl, int rg, int minb, size_t *smem, int *G) {
@@ -303,8 +316,7 @@ int apply_launch(sar_plan *pl, int rg, int minb, int Mb) {
     if (pl->d_pairs && !pair_launch(pl, rg, minb, &pair_smem, &pair_G)) return SAR_EINVAL;
     pl->pair_smem = pair_smem;
     pl->pair_G = pair_G;
-    // the largest block of the copying kernel stands for as many as fit
-    pl->mb_cap = Mb >= largest_block(pl, pl->L, minb) ? kMaxPulsesPerBlock : Mb;
+    pl->block_free = Mb == largest_block(pl, pl->L, minb) || (minb == 2 && Mb == default_block(pl, pl->L));
     pl->rg = rg;
     pl->minb = minb;
     pl->Mb = Mb;
@@ -316,8 +328,9 @@ int apply_launch(sar_plan *pl, int rg, int minb, int Mb) {
 
 // Launch shapes chosen by sar_plan_autotune, remembered for the process and
 // keyed by what the shape depends on: device, Rx count, window length,
-// storage, and max_pulses and tile count rounded up to powers of two.
-using ShapeKey = std::tuple<int, int, int, int, int, int>;
+// storage, max_pulses and tile count rounded up to powers of two, and whether
+// the plan has a pair workspace (two kernels with shapes of their own).
+using ShapeKey = std::tuple<int, int, int, int, int, int, int>;
 struct Shape {
     int rg, minb, Mb, tw;
 };
@@ -333,7 +346,7 @@ int pow2_ceil(long long v) {
 // Keyed by the plan's first tiling, whatever tiling it uses now.
 ShapeKey shape_key(const sar_plan *pl) {
     return ShapeKey{pl->device, pl->p.n_rx, pl->key_L, pl->fp16 ? 1 : 0, pow2_ceil(pl->p.max_pulses),
-                    pow2_ceil(pl->key_tiles)};
+                    pow2_ceil(pl->key_tiles), pl->d_pairs ? 1 : 0};
 }
 
 void remember_shape(const sar_plan *pl) {
@@ -594,15 +607,6 @@ int window_length(const sar_plan *pl, HostTiles &ht) {
         ti.klo_off = (float)(pl->a1 * (2.0 * ti.rho + o_allow) + pl->fd_max);
     }
     return L;
-}
-
-// Largest pulse block whose shared memory fits two CTAs per SM.
-int default_block(const sar_plan *pl, int L) {
-    const int R = pl->p.n_rx;
-    const size_t per_pulse = bp_smem_bytes(1, R, L, pl->fp16);
-    int Mb = (int)std::min<size_t>(kMaxPulsesPerBlock, std::max<size_t>(1, kBpSmemTarget / per_pulse));
-    while (Mb > 1 && bp_smem_bytes(Mb, R, L, pl->fp16) > kBpSmemTarget) --Mb;
-    return Mb;
 }
 
 // Upload a tiling and its split-tile partial sums, and make it current.  The
@@ -1119,7 +1123,7 @@ int bp_launch_pairs(sar_plan *pl, BpArgs a, cudaStream_t s, bool live) {
     pa.arrived = BpArrivals{pl->d_arrived, 0};
     pa.div_blk = ((1ull << 32) + (unsigned)a.Mb - 1) / (unsigned)a.Mb;
     pa.smem_bytes = (unsigned)pl->pair_smem;
-    pa.mb_cap = pl->mb_cap;
+    pa.mb_cap = pl->block_free ? kMaxPulsesPerBlock : pl->Mb;
     pa.polls = pl->polls;
     ExpandArgs e{};
     e.prof = a.prof;
@@ -1149,8 +1153,8 @@ int bp_launch_copying(sar_plan *pl, BpArgs a, cudaStream_t s, bool live) {
     // a call too small for the pair kernel cuts its pulse blocks so that the
     // CTAs' counts of them even out: the block that minimises, in windows'
     // time, the longest CTA (a block's set-up is worth kBlockSetup windows)
-    // plus half a window per share of a split tile.  (An explicit block stays.)
-    if (pl->mb_cap == kMaxPulsesPerBlock) {
+    // plus half a window per share of a split tile.  (A block that was set stays.)
+    if (pl->block_free) {
         long long best = INT64_MAX;
         int mb = a.Mb;
         for (int b = a.Mb; b >= 1; --b) {
@@ -1300,7 +1304,7 @@ int sar_plan_get_info(const sar_plan *pl, sar_plan_info *info) {
     i.n_tiles = pl->n_tiles;
     i.window_bins = pl->L;
     i.pulses_per_block = pl->Mb;
-    i.bp_ctas = pl->d_pairs ? pl->pair_G : pl->G;
+    i.bp_ctas = pl->G;
     i.bins_per_metre = pl->a1;
     i.cycles_per_bin = pl->beta;
     i.device_bytes = pl->used;

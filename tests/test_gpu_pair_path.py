@@ -170,3 +170,30 @@ def test_calls_on_several_streams_and_ordered_replays(M0, M1):
                 graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(img, ref[0]) and torch.equal(o, ref[1])
+
+
+@pytest.mark.parametrize("minb", [2, 3])
+def test_a_block_that_was_set_is_kept(minb):
+    """Below the line, a set block cuts the work as it cuts sar_backproject_noalloc's
+    (the same tiles split at the same chirps: the same sums, bit for bit), also
+    above the largest that fits minb CTAs per SM; that one block and a new
+    plan's leave the choice to the call."""
+    import torch
+    import paper_2306_09784_gb300 as sar
+    M = 60
+    plan, prof, qt, qr, _ = _frames(8, M, synth.Grid(-2.1, 1.2, 0.033, 0.03, 150, 130))
+    assert not plan.pair_path(M)[0]
+    lib, first = sar.load_library(), plan.launch_shape()
+    img = plan.backproject(prof, M, qt, qr)
+    most = plan.launch_shape()["pulses_per_block"]
+    assert 3 <= most <= 12
+    for mb in (1, 2, most + 1, most + 4):
+        shape = plan.set_launch(4, minb, mb)
+        assert shape["pulses_per_block"] == mb
+        ref = torch.zeros_like(img)
+        assert lib.sar_backproject_noalloc(plan.handle, prof.data_ptr(), M, qt.data_ptr(), qr.data_ptr(), None,
+                                           ref.data_ptr(), 0, torch.cuda.current_stream().cuda_stream) == sar.SAR_OK
+        assert torch.equal(plan.backproject(prof, M, qt, qr), ref), mb
+    plan.set_launch(first["rx_group"], first["regs_ctas_per_sm"], first["pulses_per_block"])
+    assert plan.launch_shape() == first
+    assert torch.equal(plan.backproject(prof, M, qt, qr), img)

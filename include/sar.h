@@ -607,6 +607,15 @@ int sar_plan_set_tile_shape(sar_plan *plan, int32_t tile_w);
 int sar_plan_pair_path(const sar_plan *plan, int32_t M, int32_t *taken, size_t *workspace_bytes);
 
 /*
+ * Gives the plan's pair workspace back (waits for the device): for a plan
+ * that only goes through batches, a server, range profiles or
+ * sar_backproject_noalloc, none of which use it.  Later sar_backproject calls
+ * take the other path.  Captured calls that took the pair path must not be
+ * replayed afterwards.  SAR_OK too when there is none.
+ */
+int sar_plan_release_pairs(sar_plan *plan);
+
+/*
  * Limit of the waits inside the kernels of later sar_backproject calls, in
  * polls (-1: the default, 2^20, far beyond any copy's time).  Kernels wait
  * for their own copies from device memory only.  A call whose wait runs out

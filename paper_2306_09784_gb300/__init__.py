@@ -34,7 +34,7 @@ EXPORTS = (
     "sar_alu_peaks", "sar_polar_grid", "sar_doppler_offsets", "sar_batch_autotune",
     "sar_batch_num_classes", "sar_batch_get_class", "sar_batch_check_errors", "sar_batch_add_frame",
     "sar_plan_set_tile_shape", "sar_plan_pair_path",
-    "sar_plan_set_wait_limit",
+    "sar_plan_set_wait_limit", "sar_plan_release_pairs",
 )
 REQ_QUEUED, REQ_RUNNING, REQ_DONE, REQ_FAILED = range(4)
 
@@ -166,6 +166,7 @@ def load_library(path: str = LIB_PATH):
     lib.sar_batch_add_frame.argtypes = [vp, vp, vp, vp, vp, i32, vp, vp, vp, i32]
     lib.sar_plan_set_tile_shape.argtypes = [vp, i32]
     lib.sar_plan_set_wait_limit.argtypes = [vp, i32]
+    lib.sar_plan_release_pairs.argtypes = [vp]
     lib.sar_plan_pair_path.argtypes = [vp, i32, ctypes.POINTER(i32), ctypes.POINTER(sz)]
     for name in EXPORTS:
         fn = getattr(lib, name)
@@ -410,6 +411,10 @@ class Plan:
         _check(self._lib.sar_plan_pair_path(self._plan, M, ctypes.byref(taken), ctypes.byref(n)),
                "sar_plan_pair_path")
         return bool(taken.value), int(n.value)
+
+    def release_pairs(self):
+        """Give the pair workspace back (a plan used only by a Batch or Server)."""
+        _check(self._lib.sar_plan_release_pairs(self._plan), "sar_plan_release_pairs")
 
     def set_wait_limit(self, polls: int = -1):
         """Polls of a kernel's wait before a call gives up (-1: the default)."""

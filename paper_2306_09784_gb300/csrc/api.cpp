@@ -68,7 +68,7 @@ struct sar_plan {
     // sums and arrival counters) and of the last Doppler offsets (partial sums):
     // a call on another stream waits (see CallOrder)
     cudaEvent_t bp_done = nullptr, doppler_done = nullptr;
-    size_t pair_smem = 0, pair_bytes = 0;
+    size_t pair_smem = 0, pair_parts[2] = {0, 0};  // bytes of the two allocations (d_call, d_pairs)
     int polls = kWaitPolls;  // of the pair kernel's waits for its copies
     int pair_G = 0;
     // Mb is the block a plan starts with (or the largest that fits minb CTAs per
@@ -235,6 +235,15 @@ int dev_alloc(sar_plan *pl, size_t bytes, void **out) {
     return SAR_OK;
 }
 
+// Gives back a dev_alloc of `bytes` (null: nothing).
+void dev_free(sar_plan *pl, void *p, size_t bytes) {
+    auto it = std::find(pl->allocs.begin(), pl->allocs.end(), p);
+    if (!p || it == pl->allocs.end()) return;
+    cudaFree(p);
+    pl->allocs.erase(it);
+    pl->used -= bytes == 0 ? 256 : (bytes + 255) & ~size_t(255);
+}
+
 template <class T>
 int upload(sar_plan *pl, const std::vector<T> &h, T **out) {
     void *p = nullptr;
@@ -313,7 +322,7 @@ int apply_launch(sar_plan *pl, int rg, int minb, int Mb) {
     if ((size_t)G * (size_t)(pl->n_tiles / G + 2) > pl->partial_slots) return SAR_EINVAL;
     size_t pair_smem = 0;
     int pair_G = 0;
-    if (pl->d_pairs && !pair_launch(pl, rg, minb, &pair_smem, &pair_G)) return SAR_EINVAL;
+    if (pl->d_pairs && !pair_launch(pl, rg, minb, &pair_smem, &pair_G)) pair_G = 0;  // not with this shape
     pl->pair_smem = pair_smem;
     pl->pair_G = pair_G;
     pl->block_free = Mb == largest_block(pl, pl->L, minb) || (minb == 2 && Mb == default_block(pl, pl->L));
@@ -745,21 +754,21 @@ void add_pair_workspace(sar_plan *pl) {
     void *small = nullptr, *pairs = nullptr;
     if (dev_alloc(pl, rx_o + geo, &small) || dev_alloc(pl, bytes, &pairs) ||
         cudaMemset(small, 0, rx_o) != cudaSuccess ||
-        cudaStreamSynchronize(nullptr) != cudaSuccess) {  // calls may come on streams that do not wait for it
+        cudaStreamSynchronize(nullptr) != cudaSuccess ||  // calls may come on streams that do not wait for it
+        !pair_launch(pl, pl->rg, pl->minb, &pl->pair_smem, &pl->pair_G)) {
         cudaGetLastError();
+        dev_free(pl, small, rx_o + geo);
+        dev_free(pl, pairs, bytes);
         return;
     }
     pl->d_pairs = (float4 *)pairs;
-    pl->pair_bytes = bytes + rx_o + geo;
     pl->d_call = (unsigned *)small;
     pl->d_zero = (float4 *)((char *)small + zero_o);
     pl->zero_len = zero_len;
     pl->d_rx = (float4 *)((char *)small + rx_o);
     pl->d_o2max = (float *)(pl->d_rx + rows);
-    if (!pair_launch(pl, pl->rg, pl->minb, &pl->pair_smem, &pl->pair_G)) {
-        pl->d_pairs = nullptr;
-        pl->pair_bytes = 0;
-    }
+    pl->pair_parts[0] = rx_o + geo;
+    pl->pair_parts[1] = bytes;
 }
 
 int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t budget, sar_plan **out) {
@@ -1097,7 +1106,7 @@ bool set_launch(const sar_plan *pl, BpArgs &a, float2 *partial, size_t slots) {
 }
 
 bool use_pairs(const sar_plan *pl, int M) {
-    return pl->d_pairs && pl->L <= pl->zero_len && pairs_pay(pl, M);
+    return pl->d_pairs && pl->pair_G > 0 && pl->L <= pl->zero_len && pairs_pay(pl, M);
 }
 
 // Backprojection from interpolation pairs of a call's arguments a.  live:
@@ -2119,7 +2128,22 @@ int sar_plan_set_tile_shape(sar_plan *pl, int32_t tile_w) {
 int sar_plan_pair_path(const sar_plan *pl, int32_t M, int32_t *taken, size_t *workspace_bytes) {
     if (!pl || !taken || M < 1 || M > pl->p.max_pulses) return SAR_EINVAL;
     *taken = use_pairs(pl, M) ? 1 : 0;
-    if (workspace_bytes) *workspace_bytes = pl->pair_bytes;
+    if (workspace_bytes) *workspace_bytes = pl->pair_parts[0] + pl->pair_parts[1];
+    return SAR_OK;
+}
+
+int sar_plan_release_pairs(sar_plan *pl) {
+    if (!pl) return SAR_EINVAL;
+    if (!pl->d_pairs) return SAR_OK;
+    DeviceGuard dg(pl->device);
+    if (!dg.ok || cudaDeviceSynchronize() != cudaSuccess) return SAR_ECUDA;
+    dev_free(pl, pl->d_call, pl->pair_parts[0]);
+    dev_free(pl, pl->d_pairs, pl->pair_parts[1]);
+    pl->d_pairs = pl->d_rx = pl->d_zero = nullptr;
+    pl->d_o2max = nullptr;
+    pl->d_call = nullptr;
+    pl->zero_len = 0;
+    pl->pair_parts[0] = pl->pair_parts[1] = 0;
     return SAR_OK;
 }
 

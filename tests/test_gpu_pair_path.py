@@ -197,3 +197,30 @@ def test_a_block_that_was_set_is_kept(minb):
     plan.set_launch(first["rx_group"], first["regs_ctas_per_sm"], first["pulses_per_block"])
     assert plan.launch_shape() == first
     assert torch.equal(plan.backproject(prof, M, qt, qr), img)
+
+
+def test_workspace_is_given_back():
+    """The memory returns to the device and to the plan's count, and calls go on
+    by the other kernel; a budget that does not hold the workspace leaves a plan
+    without it and without a part of it."""
+    import torch
+    import paper_2306_09784_gb300 as sar
+    M, grid = 1101, synth.Grid(-4.1, 1.2, 0.033, 0.03, 250, 270)
+    plan, prof, qt, qr, _ = _frames(4, M, grid)
+    taken, nbytes = plan.pair_path(M)
+    assert taken and nbytes > 0
+    before = plan.backproject(prof, M, qt, qr)
+    torch.cuda.synchronize()
+    held, free = int(plan.info.device_bytes), torch.cuda.mem_get_info()[0]
+    plan.release_pairs()
+    plan.launch_shape()  # reads the plan's info
+    assert plan.pair_path(M) == (False, 0)
+    assert held - plan.info.device_bytes >= nbytes
+    assert torch.cuda.mem_get_info()[0] >= free
+    after = plan.backproject(prof, M, qt, qr)
+    assert ((after - before).abs().norm() / before.abs().norm()).item() < 1e-5
+    plan.release_pairs()
+    left = int(plan.info.device_bytes)
+    tight = sar.Plan.from_radar(synth.Radar(n_samples=256, n_rx=4, os=4), max_pulses=M, grid=grid,
+                                crop=(plan.info.crop_lo, plan.info.crop_hi), hbm_budget=left + nbytes // 2)
+    assert tight.pair_path(M) == (False, 0) and tight.info.device_bytes == left

@@ -21,11 +21,12 @@ namespace {
 // 15 us there) and by one load in flight.
 constexpr int kMeanThreads = 256;
 
-// (e . v) / |e| with FP64 accuracy far beyond the FP32 result: 1 / |e| from an
-// FP32 reciprocal square root and one Newton step (relative error ~1e-13).  The
-// FP64 pipe has two lanes per SM: hypot and a division took ~100 of its
-// operations per distance, this takes 12.  A point on the antenna's mean
-// position has no radial direction: 0 there.
+// (e . v) / |e| in FP64: 1 / |e| from an FP32 reciprocal square root and two
+// Newton steps, as accurate as hypot and a division (the first leaves 2^-45: up
+// to 2.5e-14, which shows where the two antennas' terms cancel).  The FP64 pipe
+// has two lanes per SM: hypot and a division took ~100 of its operations per
+// distance, this takes 16.  A point on the antenna's mean position has no radial
+// direction: 0 there.
 __device__ __forceinline__ double radial(double ex, double ey, double vx, double vy) {
     const double d2 = fma(ex, ex, ey * ey), dot = fma(ex, vx, ey * vy);
     const float f = (float)d2;
@@ -36,7 +37,8 @@ __device__ __forceinline__ double radial(double ex, double ey, double vx, double
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
     const double y0 = (double)y;
-    return dot * fma(0.5 * y0, fma(-d2 * y0, y0, 1.0), y0);
+    const double y1 = fma(0.5 * y0, fma(-d2 * y0, y0, 1.0), y0);
+    return dot * fma(0.5 * y1, fma(-d2 * y1, y1, 1.0), y1);
 }
 
 // sums[cta][0..5]: this CTA's share of the sums of (q_tx.x, q_tx.y, q_rx.x,

@@ -893,7 +893,7 @@ int plan_create(const sar_radar_params *params, const sar_grid *grid, size_t bud
     // inter-pass twiddles and the output coefficients
     std::vector<float4> rc_pre2, rc_cmb;
     std::vector<float2> rc_twd2;
-    pl->rc_band = pl->rc_split ? rc_band_mask(p.n_samples, p.os, pl->crop_lo, pl->crop_hi) : 0;
+    pl->rc_band = pl->rc_split ? rc_band_mask(p.n_samples, p.os, pl->crop_lo, pl->crop_hi, pl->fp16) : 0;
     if (pl->rc_band) {
         const int N = p.n_samples, D = N / 256, ho = p.os / 2, RT = 16 * D * ho;
         rc_pre2.resize((size_t)16 * RT);

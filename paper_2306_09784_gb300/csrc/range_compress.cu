@@ -1089,10 +1089,17 @@ int rc_rows_per_group(const RcSplitArgs &a) { return kSplitThreads / (a.N2 * a.o
 
 // The band kernel's mask of 16-value blocks of Y, or 0 where the kernel does not
 // apply: at most 256 values of Q (else a block of Y serves several), sizes where
-// it is the faster one (see the kernel).
-unsigned rc_band_mask(int n_samples, int os, int crop_lo, int crop_hi) {
+// it is the faster one (see the kernel).  At N = 512 a bin costs two complex
+// products there, which wide crops feel from os = 8 on: 8192 rows, os 16, FP32,
+// band against split kernel: 176 os bins 150-159 us against 155-160, 192 os 154-164
+// against 156-158, 255 os 172-183 against 170-172; FP16, which the split kernel
+// stores at more cost: 224 os 189-198 against 194-197, 255 os 204-211 against
+// 205-206.  N = 256 gains 17-32 % up to its whole spectrum, N = 512 with os 4
+// 0-15 %.
+unsigned rc_band_mask(int n_samples, int os, int crop_lo, int crop_hi, bool fp16) {
     if (!rc_split_supported(n_samples, os) || os < 4 || n_samples > 512 || n_samples * os > 8192) return 0;
     if (crop_hi / os - crop_lo / os >= 256) return 0;
+    if (n_samples == 512 && os >= 8 && crop_hi - crop_lo + 1 > (fp16 ? 232 : 184) * os) return 0;
     unsigned mask = 0;
     for (int q = crop_lo / os; q <= crop_hi / os; ++q) mask |= 1u << ((q & 255) >> 4);
     return mask;

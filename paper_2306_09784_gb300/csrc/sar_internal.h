@@ -74,7 +74,7 @@ struct RcSplitBatch {
     int n_jobs;
 };
 bool rc_split_supported(int n_samples, int os);
-unsigned rc_band_mask(int n_samples, int os, int crop_lo, int crop_hi);
+unsigned rc_band_mask(int n_samples, int os, int crop_lo, int crop_hi, bool fp16);
 int rc_rows_per_group(const RcSplitArgs &a);
 // tab == null: the single job a; otherwise a gives N2 and os of the table's
 // jobs and groups is the table's total row-group count.

@@ -70,3 +70,17 @@ def test_batch_of_band_and_split_frames(precision):
         assert torch.equal(_values(plan, prof, M, 2, precision), _values(plan, alone, M, 2, precision))
         ref = plan.backproject(alone, M, qt, qr)
         assert ((img - ref).abs().norm() / ref.abs().norm()).item() < 1e-5
+
+
+@pytest.mark.parametrize("N,os_f", [(256, 1), (256, 2), (256, 4), (256, 8), (512, 1), (1024, 16)])
+@pytest.mark.parametrize("sign", [1, -1])
+def test_spectrum_on_each_kernel(N, os_f, sign):
+    import torch
+    import paper_2306_09784_gb300 as sar
+    radar = synth.Radar(n_samples=N, n_rx=2, os=os_f)
+    plan = sar.Plan.from_radar(radar, max_pulses=33, grid=synth.Grid(-1.0, 2.0, 0.05, 0.05, 8, 8), crop=(2, 40),
+                               phase_sign=sign)
+    beat = torch.randn(33, 2, N, dtype=torch.complex64, device="cuda", generator=torch.Generator("cuda").manual_seed(N))
+    S, _ = _reference(radar, beat, sign, (2, 40))
+    got = plan.range_spectrum(beat).to(torch.complex128)
+    assert ((got - S).abs().square().sum(-1).sqrt() / S.abs().square().sum(-1).sqrt()).max().item() <= 1e-6

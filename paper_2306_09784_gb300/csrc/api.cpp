@@ -34,6 +34,8 @@ constexpr unsigned kCallSlots = 1024;
 // of L bins, and spends, against the copying kernel (see pairs_pay).
 constexpr double kPairPerWindow = 52.0, kPairPerWindowBin = 3.8, kPairPerPulseTile = 365.0;
 constexpr double kPairPerCall = 12.0e6, kPairPerTile = 3.5e3, kPairPerRowBin = 7.4;
+// Bins of pairs that the L2 cache holds (128 MB); beyond it each costs as much again.
+constexpr double kPairRowBinsL2 = 8.0e6;
 // Set-up of a pulse block of the copying kernel, in windows' time (~1 us, 12 of
 // ~70 ns): 128 x 128 x 256 x 1 frame 24.6 us at blocks of 16 or 32 chirps, 28.7
 // at 24, where the last CTAs of a second round run alone.
@@ -703,30 +705,32 @@ size_t profile_bytes(const sar_plan *pl, int M) {
 // tiling).  Against the copying kernel it saves the conversion of every window's
 // bins and some set-up per (window, Rx), and it spends an expansion of whole
 // profile rows, reach word and launch per call, set-up per tile, and more per
-// (tile, chirp) than a single Rx gives back.  The six figures are a fit to 400
+// (tile, chirp) than a single Rx gives back.  The figures are a fit to 400
 // calls timed on both kernels (24 to 2600 pixels a side, 1 to 4096 chirps, 1 to
 // 16 Rx, 38 to 4096 bins, windows of 20 to 132): the rule's choice is 0.3 %
 // slower than the faster kernel on average, and at worst 5 % slower than the
-// copying kernel.  1024 chirps x 4 Rx on 256 tiles: 817 us against 884; 64 x 64
+// copying kernel (one call; the next 2 %).  1024 chirps x 4 Rx on 256 tiles: 817 us against 884; 64 x 64
 // pixels, 16384 chirps of 2048 bins each: 279 us against 99, not taken; 2048 x
 // 2048 pixels, 16 chirps: 154 against 107, not taken; one Rx, windows of 20
 // bins, 2298 chirps on 275 tiles: 757 against 733, not taken.
 bool pairs_pay(const sar_plan *pl, int M) {
     const double rows = (double)M * pl->p.n_rx, windows = rows * pl->n_tiles;
     const double saved = windows * (kPairPerWindow + kPairPerWindowBin * pl->L - kPairPerPulseTile / pl->p.n_rx);
-    return saved > kPairPerCall + kPairPerTile * pl->n_tiles + kPairPerRowBin * rows * pl->n_bins;
+    const double bins = rows * pl->n_bins, far_bins = std::max(0.0, bins - kPairRowBinsL2);
+    return saved > kPairPerCall + kPairPerTile * pl->n_tiles + kPairPerRowBin * (bins + far_bins);
 }
 
 // Workspace of the pair kernel: 16 bytes per bin of max_pulses chirps, twice
 // an FP32 profile buffer.  A plan goes without (and uses the copying kernel)
 // where no call of its size takes that path (what a call saves less what it
-// spends grows with its chirps), where it would take more than 1 GiB or a
-// sixteenth of the free memory, or where an HBM budget would then no longer
-// hold the buffers that sar_form_image_host and sar_plan_set_tile_shape
-// allocate later.
+// spends is greatest at its most chirps or where its pairs just fit L2), where
+// it would take more than 1 GiB or a sixteenth of the free memory, or where an
+// HBM budget would then no longer hold the buffers that sar_form_image_host and
+// sar_plan_set_tile_shape allocate later.
 void add_pair_workspace(sar_plan *pl) {
     const size_t rows = (size_t)pl->p.max_pulses * pl->p.n_rx;
-    if (!pairs_pay(pl, pl->p.max_pulses)) return;
+    const int fit = (int)std::min<double>(pl->p.max_pulses, kPairRowBinsL2 / ((double)pl->p.n_rx * pl->n_bins));
+    if (!pairs_pay(pl, pl->p.max_pulses) && !pairs_pay(pl, std::max(1, fit))) return;
     const size_t bytes = rows * pl->n_bins * sizeof(float4);
     const size_t geo = rows * sizeof(float4) + (size_t)pl->p.max_pulses * sizeof(float);
     size_t free_b = 0, total_b = 0;

@@ -224,3 +224,11 @@ def test_workspace_is_given_back():
     tight = sar.Plan.from_radar(synth.Radar(n_samples=256, n_rx=4, os=4), max_pulses=M, grid=grid,
                                 crop=(plan.info.crop_lo, plan.info.crop_hi), hbm_budget=left + nbytes // 2)
     assert tight.pair_path(M) == (False, 0) and tight.info.device_bytes == left
+
+
+def test_workspace_for_calls_whose_pairs_fit_l2():
+    """A plan whose largest call does not gain, as its pairs leave the L2 cache,
+    has a workspace all the same when its shorter calls gain."""
+    for n_rx, side, bins, short, M in ((4, (320, 320), 1024, 1400, 8000), (6, (288, 1024), 2048, 640, 1156)):
+        plan = _plan(n_rx, M, *side, spacing=0.025 if n_rx == 4 else 0.01, bins=bins)
+        assert [plan.pair_path(m)[0] for m in (short, M)] == [True, False] and plan.pair_path(short)[1] > 0

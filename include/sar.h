@@ -234,7 +234,7 @@ int sar_range_compress(sar_plan *plan, const void *beat_dev, int32_t M,
 
 /*
  * The plain windowed, zero-padded range transform S[m][r][k] for all
- * k < N_fft as complex64 [M][R][N_fft] (same transforms as sar_range_compress,
+ * k < N_fft as complex64 [M][R][N_fft] (the transform of sar_range_compress,
  * without window w_sar, rotation or crop).  For inspection and parity checks.
  */
 int sar_range_spectrum(sar_plan *plan, const void *beat_dev, int32_t M,

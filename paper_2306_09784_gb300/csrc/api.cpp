@@ -1211,9 +1211,11 @@ struct CallOrder {
         done = last;
         s = stream;
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return false;
+        bool ok = cudaStreamIsCapturing(s, &cap) == cudaSuccess;
         live = cap == cudaStreamCaptureStatusNone;
-        return !live || cudaStreamWaitEvent(s, done, 0) == cudaSuccess;
+        if (ok && live) ok = cudaStreamWaitEvent(s, done, 0) == cudaSuccess;
+        if (!ok) cudaGetLastError();  // refused here (the legacy stream beside a capture): not the next call's error
+        return ok;
     }
     bool end() const { return !live || cudaEventRecord(done, s) == cudaSuccess; }
 };

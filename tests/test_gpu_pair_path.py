@@ -232,3 +232,35 @@ def test_workspace_for_calls_whose_pairs_fit_l2():
     for n_rx, side, bins, short, M in ((4, (320, 320), 1024, 1400, 8000), (6, (288, 1024), 2048, 640, 1156)):
         plan = _plan(n_rx, M, *side, spacing=0.025 if n_rx == 4 else 0.01, bins=bins)
         assert [plan.pair_path(m)[0] for m in (short, M)] == [True, False] and plan.pair_path(short)[1] > 0
+
+
+def test_a_refused_call_leaves_no_error_behind():
+    """A call on the legacy stream beside the capture of a blocking stream is
+    refused; the same call after the capture is a call like any other."""
+    import ctypes
+
+    import torch
+    import paper_2306_09784_gb300 as sar
+    M = 600
+    plan, prof, qt, qr, _ = _frames(4, M, synth.Grid(-4.1, 1.2, 0.033, 0.03, 250, 270))
+    assert plan.pair_path(M)[0]
+    ref = plan.backproject(prof, M, qt, qr)
+    torch.cuda.synchronize()
+    cu, lib = ctypes.CDLL("libcuda.so.1"), sar.load_library()
+    stream, graph, img = ctypes.c_void_p(), ctypes.c_void_p(), torch.zeros_like(ref)
+
+    def call():
+        return lib.sar_backproject(plan.handle, prof.data_ptr(), M, qt.data_ptr(), qr.data_ptr(), None, img.data_ptr(),
+                                   0, None)
+
+    torch.cuda.synchronize()
+    assert cu.cuStreamCreate(ctypes.byref(stream), 0) == 0
+    assert cu.cuStreamBeginCapture_v2(stream, 2) == 0  # relaxed: only this stream's own work is captured
+    refused = call()
+    assert cu.cuStreamEndCapture(stream, ctypes.byref(graph)) == 0
+    assert refused == sar.SAR_ECUDA
+    assert call() == sar.SAR_OK
+    torch.cuda.synchronize()
+    assert torch.equal(img, ref) and plan.check_errors() == sar.SAR_OK
+    cu.cuGraphDestroy(graph)
+    cu.cuStreamDestroy_v2(stream)
